@@ -17,10 +17,10 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libshacsim.so")
 SOURCES = ["shac_api.cu", "shac_kernels.cu", "shac_learner.cu", "shac_jit.cu"]
-HEADERS = ["shac_device.cuh", "shac_kernels.cuh", "shac_batched.cuh", "shac_jit.h"]
+HEADERS = ["shac_device.cuh", "shac_kernels.cuh", "shac_team.cuh", "shac_batched.cuh", "shac_jit.h"]
 # device sources compiled again at run time, embedded as string constants
 EMBEDDED = [("shac_jit_src_device", "shac_device.cuh"), ("shac_jit_src_kernels", "shac_kernels.cuh"),
-            ("shac_jit_src_batched", "shac_batched.cuh")]
+            ("shac_jit_src_team", "shac_team.cuh"), ("shac_jit_src_batched", "shac_batched.cuh")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 

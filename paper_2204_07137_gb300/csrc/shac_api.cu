@@ -10,6 +10,7 @@
 #include "../../include/shacsim.h"
 #include "shac_jit.h"
 #include "shac_kernels.cuh"
+#include "shac_team.cuh"
 
 using namespace shac;
 
@@ -20,16 +21,17 @@ struct shac_model {
   int height_q = -1, vx_dof = -1;   // reward / termination coordinates (free root: 2 / world vx)
   std::vector<int> parent, jtype, qs, ds, nd, lvl_ptr, lvl_link, ch_ptr, ch_idx, lc_ptr, lc_idx, lm_ptr, lm_idx, dof_link,
       dof_k,
-      dof_act, item_link, seg_mus, mus_seg_ptr, anc_mask, chain_tail;
-  std::vector<float> axis, jpos, jrot, mass, com, icom, qlo, qhi, arm, damp, gear, item_pos, crad, fmax, rwq, rwqd;
-  DevModel layout;   // sizes + scratch offsets (pointers unset)
+      dof_act, item_link, seg_mus, mus_seg_ptr, anc_mask, chain_tail, ln_i, ms_ptr, sg_place;
+  std::vector<float> axis, jpos, jrot, mass, com, icom, qlo, qhi, arm, damp, gear, item_pos, crad, fmax, rwq, rwqd, ln_f, sg_f;
+  int lanes_needed = 0, nround = 0, mrows = 0;
+  DevModel layout, lane_layout;   // sizes + scratch offsets (pointers unset): general and lane form
 };
 
 struct Group {
   const shac_model* m;
   int N;
   void* blob = nullptr;      // device copy of the model arrays
-  DevModel dev;              // with device pointers
+  DevModel dev, lane_dev;    // with device pointers: general and lane layouts
   int lanes = 0;             // batched team size
 };
 
@@ -40,7 +42,7 @@ struct shac_batch {
   int warps_per_cta = 4;
   int64_t q_size = 0, qd_size = 0, act_size = 0, n_envs = 0;
   IOArgs io{};
-  DevModel* d_models = nullptr;
+  DevModel* d_models = nullptr;        // [n_groups] general layouts, then [n_groups] lane layouts
   unsigned int* d_flags = nullptr;
   WorkItem* d_items = nullptr;
   int n_items = 0;
@@ -74,6 +76,109 @@ static void quat_rot(const float* q, float* R) {
   for (int i = 0; i < 9; ++i) R[i] = (float)r[i];
 }
 
+// Row capacity of the register dense path (shac_device.cuh) that holds nv rows.
+static int dense_rows(int nv) {
+  static const int sizes[] = {2, 4, 6, 8, 10, 12, 14, 16, 20, 24, 28, 32};
+  for (int nm : sizes)
+    if (nm >= nv) return nm;
+  return 32;
+}
+
+// Columns of the muscles' via-point items (shac_team.cuh): the fewest rows for
+// which every link's items fit in columns of its own.
+static void compute_muscle_slots(shac_model* m) {
+  const int L = m->L;
+  m->mrows = 0;
+  m->ms_ptr.assign(L + 1, 0);
+  if (m->nseg == 0 || m->lanes_needed > LANE_COLS) return;
+  auto columns = [&](int rows) {
+    int n = 0;
+    for (int i = 0; i < L; ++i) n += (m->lm_ptr[i + 1] - m->lm_ptr[i] + rows - 1) / rows;
+    return n;
+  };
+  m->mrows = (2 * m->nseg + MSLOTS - 1) / MSLOTS;
+  while (columns(m->mrows) > MSLOTS) ++m->mrows;   // ends: a column per link suffices, and L <= MSLOTS
+  std::vector<int> place(m->nitems, 0);
+  int s = 0;
+  for (int i = 0; i < L; ++i) {
+    m->ms_ptr[i] = s;
+    const int n = m->lm_ptr[i + 1] - m->lm_ptr[i];
+    for (int k = 0; k < n; ++k) place[m->lm_idx[m->lm_ptr[i] + k]] = (k % m->mrows) * MSLOTS + s + k / m->mrows;
+    s += (n + m->mrows - 1) / m->mrows;
+  }
+  m->ms_ptr[L] = s;
+  m->sg_f.assign((size_t)8 * m->nseg, 0.f);
+  m->sg_place.assign(m->nseg, 0);
+  for (int g = 0; g < m->nseg; ++g) {
+    const int e0 = m->nc + 2 * g, e1 = e0 + 1;
+    const unsigned id = (unsigned)m->item_link[e0] | (unsigned)m->item_link[e1] << 8 | (unsigned)m->seg_mus[g] << 16;
+    for (int k = 0; k < 3; ++k) {
+      m->sg_f[4 * g + k] = m->item_pos[3 * e0 + k];
+      m->sg_f[4 * (m->nseg + g) + k] = m->item_pos[3 * e1 + k];
+    }
+    m->sg_f[4 * g + 3] = m->fmax[m->seg_mus[g]];
+    std::memcpy(&m->sg_f[4 * (m->nseg + g) + 3], &id, sizeof id);
+    m->sg_place[g] = place[e0] | place[e1] << 16;
+  }
+}
+
+// Lane columns of the model (shac_team.cuh): lane d owns DOF d, and the link
+// whose first DOF it is; links without a DOF take the lanes from nv on.  More
+// than 32 lanes needed: the model has no lane form.
+static void compute_lanes(shac_model* m) {
+  const int L = m->L, nv = m->nv;
+  std::vector<int> lane_of(L), level(L, 0);
+  int next = nv, deepest = 0;
+  for (int i = 0; i < L; ++i) {
+    lane_of[i] = m->nd[i] > 0 ? m->ds[i] : next++;
+    if (m->parent[i] >= 0) level[i] = level[m->parent[i]] + 1;
+    deepest = std::max(deepest, level[i]);
+  }
+  m->lanes_needed = next;
+  compute_muscle_slots(m);
+  m->nround = 0;
+  while ((1 << m->nround) < deepest + 1) ++m->nround;
+  m->ln_i.assign(LI_N * LANE_COLS, 0);
+  m->ln_f.assign(LF_N * LANE_COLS, 0.f);
+  if (next > LANE_COLS) return;
+  auto I = [&](int f, int lane) -> int& { return m->ln_i[f * LANE_COLS + lane]; };
+  auto F = [&](int f, int lane) -> float& { return m->ln_f[f * LANE_COLS + lane]; };
+  for (int l = 0; l < LANE_COLS; ++l) {   // lanes without a link: an identity rotation, no ancestors
+    I(LI_LINK, l) = -1; I(LI_JT, l) = J_FIXED; I(LI_ANC, l) = (1 << 30) - 1; I(LI_ACT, l) = -1;
+    F(LF_JROT, l) = F(LF_JROT + 4, l) = F(LF_JROT + 8, l) = 1.f;
+    F(LF_ARM, l) = 1.f;                   // identity rows below nv
+  }
+  for (int i = 0; i < L; ++i) {
+    const int l = lane_of[i];
+    I(LI_LINK, l) = i; I(LI_JT, l) = m->jtype[i]; I(LI_Q, l) = m->qs[i];
+    I(LI_C0, l) = m->lc_ptr[i]; I(LI_C1, l) = m->lc_ptr[i + 1];
+    I(LI_BASE, l) = m->parent[i] < 0;
+    unsigned anc = 0;                     // the 2^r-th ancestors' lanes, 6 bits each (63: none)
+    for (int r = 0; r < 5; ++r) {
+      int j = i;
+      for (int k = 0; k < (1 << r) && j >= 0; ++k) j = m->parent[j];
+      anc |= (unsigned)(j >= 0 ? lane_of[j] : 63) << (6 * r);
+    }
+    I(LI_ANC, l) = (int)anc;
+    for (int k = 0; k < 3; ++k) {
+      F(LF_AXIS + k, l) = m->axis[3 * i + k];
+      F(LF_JPOS + k, l) = m->jpos[3 * i + k];
+      F(LF_COM + k, l) = m->com[3 * i + k];
+    }
+    for (int k = 0; k < 9; ++k) F(LF_JROT + k, l) = m->jrot[9 * i + k];
+    for (int k = 0; k < 6; ++k) F(LF_ICOM + k, l) = m->icom[6 * i + k];
+    F(LF_MASS, l) = m->mass[i];
+  }
+  for (int d = 0; d < nv; ++d) {
+    I(LI_DLINK, d) = m->dof_link[d];
+    I(LI_ACT, d) = m->dof_act[d];
+    for (int a = 0; a < nv; ++a)          // DOF a moves with d: an entry of d's row of the upper triangle
+      if (((unsigned)m->anc_mask[a] >> d) & 1u) I(LI_DESC, d) |= (int)(1u << a);
+    F(LF_ARM, d) = m->arm[d]; F(LF_DAMP, d) = m->damp[d]; F(LF_GEAR, d) = m->gear[d];
+    F(LF_QLO, d) = m->qlo[d]; F(LF_QHI, d) = m->qhi[d];
+  }
+}
+
 static void compute_layout(shac_model* m) {
   DevModel& d = m->layout;
   std::memset(&d, 0, sizeof(d));
@@ -97,6 +202,9 @@ static void compute_layout(shac_model* m) {
   d.rec_floats = o;
   take(d.o_ACT, m->na); take(d.o_QB, m->nq); take(d.o_QDB, nv); take(d.o_ACTB, m->na);
   take(d.o_QC, m->nq); take(d.o_QDC, nv); take(d.o_LW, LWORK * L);
+  d.lanes_needed = m->lanes_needed;
+  d.nround = m->nround;
+  d.mrows = m->mrows;
   take(d.o_B, nv); take(d.o_T, nv);
   take(d.o_LAM, nv); take(d.o_ITB, 10 * ni);
   take(d.o_SEGA, m->nseg);
@@ -108,6 +216,29 @@ static void compute_layout(shac_model* m) {
   // 6 floats forward, 12 in reverse
   take(d.o_MW, m->nseg > 0 ? std::max(32, L) * 12 : 0);
   d.env_floats = o;
+
+  // Lane form: the state and the per-link quantities live in registers, so the
+  // scratch holds what steps exchange with the caller's buffers, the exchange
+  // buffers and one record's copy (and for muscles the poses, force cotangents
+  // and items their segments share).  Without muscles its records are never
+  // longer than the general ones.
+  DevModel& l = m->lane_layout;
+  l = d;
+  o = 0;
+  take(l.o_Q, m->nq); take(l.o_QD, nv); take(l.o_ACT, m->na); take(l.o_QB, m->nq); take(l.o_QDB, nv);
+  take(l.o_ACTB, m->na);
+  take(l.o_QC, m->nq); take(l.o_QDC, nv);
+  if (m->nseg > 0) {
+    take(l.o_SEGA, m->nseg); take(l.o_MW, 12 * MSLOTS); take(l.o_MB, 6 * L);
+    o = (o + 3) / 4 * 4;
+    take(l.o_MP, 12 * L); take(l.o_MX, 3 * MSLOTS * m->mrows); take(l.o_MF, 3 * MSLOTS * m->mrows);
+  }
+  o = (o + 3) / 4 * 4;
+  const LaneRecord rec = lane_record(L, nv, dense_rows(nv), m->root_free);
+  take(l.o_X, (lane_xchg_floats(L, dense_rows(nv)) + 3) / 4 * 4);
+  take(l.o_R, rec.items);
+  l.env_floats = o;
+  l.rec_floats = rec.items + 3 * MSLOTS * m->mrows;
 }
 
 extern "C" shac_status shac_model_create(const shac_model_desc* dsc, shac_model** out) {
@@ -275,6 +406,7 @@ extern "C" shac_status shac_model_create(const shac_model_desc* dsc, shac_model*
   m->rwq.assign(dsc->rw_q, dsc->rw_q + nq);
   m->rwqd.assign(dsc->rw_qd, dsc->rw_qd + nv);
   for (int k = 0; k < 10; ++k) m->rc[k] = dsc->reward_coef[k];
+  compute_lanes(m);
   compute_layout(m);
   *out = m;
   return SHAC_OK;
@@ -318,6 +450,9 @@ static shac_status upload_model(const shac_model* m, Group& g) {
     addi(&tmp, m->anc_mask);
     ifix.back().first = reinterpret_cast<const int**>(&d.anc_mask);
   }
+  addi(&d.ln_i, m->ln_i); addi(&d.ms_ptr, m->ms_ptr); addi(&d.sg_place, m->sg_place);
+  addf(&d.sg_f, m->sg_f);   // first: read 16 bytes at a time
+  addf(&d.ln_f, m->ln_f);
   addf(&d.axis, m->axis); addf(&d.jpos, m->jpos); addf(&d.jrot, m->jrot); addf(&d.mass, m->mass); addf(&d.com, m->com);
   addf(&d.icom, m->icom); addf(&d.qlo, m->qlo); addf(&d.qhi, m->qhi); addf(&d.arm, m->arm); addf(&d.damp, m->damp);
   addf(&d.gear, m->gear); addf(&d.item_pos, m->item_pos); addf(&d.crad, m->crad); addf(&d.fmax, m->fmax);
@@ -333,6 +468,14 @@ static shac_status upload_model(const shac_model* m, Group& g) {
   for (auto& f : ifix) *f.first = reinterpret_cast<const int*>(dev) + f.second;
   for (auto& f : ffix) *f.first = reinterpret_cast<const float*>(dev + ibytes) + f.second;
   g.blob = dev;
+  g.lane_dev = g.dev;   // the same arrays under the lane form's offsets
+  const DevModel& l = m->lane_layout;
+  int DevModel::*const offsets[] = {&DevModel::o_Q, &DevModel::o_QD, &DevModel::o_ACT, &DevModel::o_QB, &DevModel::o_QDB,
+                                    &DevModel::o_ACTB, &DevModel::o_QC, &DevModel::o_QDC, &DevModel::o_SEGA,
+                                    &DevModel::o_MW, &DevModel::o_X, &DevModel::o_R, &DevModel::o_MP, &DevModel::o_MB,
+                                    &DevModel::o_MX, &DevModel::o_MF, &DevModel::rec_floats,
+                                    &DevModel::env_floats};
+  for (int DevModel::*f : offsets) g.lane_dev.*f = l.*f;
   return SHAC_OK;
 }
 
@@ -350,24 +493,39 @@ static int default_lanes(const shac_model* m) {
 // nv rows, one padded row per lane, when the team has that many lanes; 0
 // selects the shared-memory form.
 static int dense_class(int nv, int lanes) {
-  static const int sizes[] = {2, 4, 6, 8, 10, 12, 14, 16, 20, 24, 28, 32};
-  for (int nm : sizes)
-    if (nm >= nv) return nm <= lanes ? nm : 0;
-  return 0;
+  const int nm = dense_rows(nv);
+  return nm <= lanes ? nm : 0;
+}
+
+// Whether group g's team covers its links and DOFs with a lane each
+// (shac_team.cuh) and its records fit the workspace, which is laid out for the
+// general ones (a handful of muscles may not: their items come in whole rows);
+// a batch takes the lane kernels when all its groups do.
+static bool lane_form(const Group& g) {
+  return g.N == 0 || (g.m->lanes_needed <= g.lanes && dense_class(g.m->nv, g.lanes) > 0 &&
+                      g.m->lane_layout.rec_floats <= g.m->layout.rec_floats);
+}
+static bool lane_form(const shac_batch* b) {
+  for (const Group& g : b->groups)
+    if (!lane_form(g)) return false;
+  return true;
 }
 
 // Shared floats per environment: padded so that every environment's scratch
 // starts 16-byte aligned (records move 16 bytes at a time) and the 32 / lanes
 // teams of a warp start spread over the 32 banks (lanes apart, at least 4).
-static int env_stride(const shac_model* m, int lanes) {
-  return ((m->layout.env_floats + 31) / 32) * 32 + (lanes >= 4 ? lanes % 32 : 4);
+static int env_stride(const DevModel& layout, int lanes) {
+  return ((layout.env_floats + 31) / 32) * 32 + (lanes >= 4 ? lanes % 32 : 4);
+}
+static const DevModel& batch_layout(const shac_batch* b, const Group& g) {
+  return lane_form(b) ? g.m->lane_layout : g.m->layout;
 }
 
 static size_t batched_smem_warp_floats(const shac_batch* b) {
   size_t per_warp = 0;
   for (const Group& g : b->groups) {
     if (g.N == 0) continue;
-    per_warp = std::max(per_warp, (size_t)(32 / g.lanes) * env_stride(g.m, g.lanes));
+    per_warp = std::max(per_warp, (size_t)(32 / g.lanes) * env_stride(batch_layout(b, g), g.lanes));
   }
   return per_warp;
 }
@@ -479,6 +637,7 @@ extern "C" shac_status shac_batch_create(const shac_model* const* models, const 
   b->io.q_size = b->q_size; b->io.qd_size = b->qd_size; b->io.act_size = b->act_size; b->io.n_envs = b->n_envs;
   std::vector<DevModel> dm;
   for (auto& g : b->groups) dm.push_back(g.dev);
+  for (auto& g : b->groups) dm.push_back(g.lane_dev);
   if (cudaMalloc(&b->d_models, dm.size() * sizeof(DevModel)) != cudaSuccess ||
       cudaMemcpy(b->d_models, dm.data(), dm.size() * sizeof(DevModel), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMalloc(&b->d_flags, sizeof(unsigned int)) != cudaSuccess ||
@@ -553,8 +712,9 @@ extern "C" shac_status shac_batch_specialize(shac_batch* b, int32_t enable) {
   if (dev != b->device) return SHAC_ERR_INVALID_ARG;
   const Group& g = b->groups[0];
   JitKernels k;
-  const shac_status st = jit_kernels(b->device, g.m->layout, g.m->parent, g.lanes, dense_class(g.m->nv, g.lanes),
-                                     env_stride(g.m, g.lanes), &k, nullptr);
+  const shac_status st = jit_kernels(b->device, batch_layout(b, g), g.m->parent, g.m->anc_mask, g.lanes,
+                                     dense_class(g.m->nv, g.lanes), env_stride(batch_layout(b, g), g.lanes), lane_form(b),
+                                     &k, nullptr);
   if (st != SHAC_OK) return st;
   b->spec = k;
   b->spec_lanes = g.lanes;
@@ -581,12 +741,13 @@ static PlainGroup plain_group(const shac_batch* b, int gi, void* ws) {
 
 static shac_status batched_launch(shac_batch* b, BatchedArgs& a, void* ws, cudaStream_t s, bool adjoint,
                                   bool window = false) {
-  a.models = b->d_models;
+  const bool lanes = lane_form(b);
+  a.models = b->d_models + (lanes ? b->groups.size() : 0);
   a.n_groups = (int)b->groups.size();
   a.io = b->io;
   for (int gi = 0; gi < a.n_groups; ++gi) {
     a.lanes[gi] = b->groups[gi].lanes;
-    a.env_stride[gi] = env_stride(b->groups[gi].m, b->groups[gi].lanes);
+    a.env_stride[gi] = env_stride(batch_layout(b, b->groups[gi]), b->groups[gi].lanes);
     a.dense_nm[gi] = dense_class(b->groups[gi].m->nv, b->groups[gi].lanes);
   }
   a.smem_warp_floats = (int)batched_smem_warp_floats(b);
@@ -619,12 +780,12 @@ static shac_status batched_launch(shac_batch* b, BatchedArgs& a, void* ws, cudaS
   // the kernels' static part (the model table) is under 8 KB.
   if (smem > 40 * 1024) {
     const cudaError_t e = spec ? cudaFuncSetAttribute(spec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                               : batched_set_smem_limit(smem);
+                               : batched_set_smem_limit(smem, lanes);
     if (e != cudaSuccess) return SHAC_ERR_CAPACITY;
   }
   int occ = 0;
   const cudaError_t oe = spec ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, spec, block, smem)
-                              : batched_occupancy(&occ, block, smem, adjoint);
+                              : batched_occupancy(&occ, block, smem, adjoint, lanes);
   if (oe != cudaSuccess) return SHAC_ERR_CUDA;
   if (occ < 1) return SHAC_ERR_CAPACITY;
   const int grid = std::max(1, std::min(b->num_sms * occ, (b->n_items + W - 1) / W));
@@ -633,8 +794,8 @@ static shac_status batched_launch(shac_batch* b, BatchedArgs& a, void* ws, cudaS
     void* args[] = {&a};
     return cuda_ok(cudaLaunchKernel(spec, dim3(grid), dim3(block), args, smem, s));
   }
-  if (adjoint) launch_batched_adjoint(a, grid, block, smem, s);
-  else launch_batched_forward(a, grid, block, smem, s);
+  if (adjoint) launch_batched_adjoint(a, grid, block, smem, lanes, s);
+  else launch_batched_forward(a, grid, block, smem, lanes, s);
   return cuda_ok(cudaGetLastError());
 }
 

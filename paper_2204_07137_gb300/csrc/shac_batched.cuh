@@ -9,6 +9,7 @@
 // address arithmetic and the loop bounds they control.
 #pragma once
 #include "shac_kernels.cuh"
+#include "shac_team.cuh"
 
 // Launch-shape values of a specialised build (the generic build reads them
 // from the launch arguments).
@@ -26,10 +27,10 @@ namespace shac {
 
 // Register caps of the batched kernels (forward, adjoint): the live state of
 // the chain carries and of the 32-row dense path fits without spills; the
-// host launches at most 8 warps per CTA (8 x 32 x 216 registers fit an SM's
+// host launches at most 8 warps per CTA (8 x 32 x 240 registers fit an SM's
 // 64 Ki, and two 4-warp CTAs stay resident per SM).
-#define BATCHED_REGS_FORWARD 184
-#define BATCHED_REGS_ADJOINT 216
+#define BATCHED_REGS_FORWARD 208
+#define BATCHED_REGS_ADJOINT 240
 
 
 struct Team {
@@ -74,7 +75,9 @@ __device__ __forceinline__ void record_save(float* dst, const SMem& w, int n, in
   for (int j = lane; j < n / 4; j += nl) d4[j] = s4[j];
 }
 
-// One work item of the forward window (all steps, all substeps).
+// One work item of the forward window (all steps, all substeps).  LANES: the
+// lane form of the substep (the team has a lane per link and DOF).
+template <bool LANES>
 __device__ __forceinline__ void forward_item(const BatchedArgs& a, const DevModel& M, const WorkItem& it,
                                              const SMem& w, const Team& t) {
   const int nm = SHAC_DENSE_ROWS(a.dense_nm[it.group]);
@@ -84,6 +87,12 @@ __device__ __forceinline__ void forward_item(const BatchedArgs& a, const DevMode
   if (a.q_copy0) {
     team_store(w, M.o_Q, a.q_copy0 + io.q_off, M.nq, io.N, t.env, t.lane, t.nl, t.active);
     team_store(w, M.o_QD, a.qd_copy0 + io.qd_off, M.nv, io.N, t.env, t.lane, t.nl, t.active);
+  }
+  LaneConst lc;
+  LaneState ls;
+  if (LANES) {
+    lc = lane_const(M, t.lane);
+    if (M.nseg > 0) muscle_clear(M, w, t.lane, t.nl);
   }
   int ep = 0;   // episodic window: steps since the last reset (team lane 0)
   if (a.done && t.lane == 0) ep = a.ep_step[io.env_off + t.env];
@@ -96,7 +105,15 @@ __device__ __forceinline__ void forward_item(const BatchedArgs& a, const DevMode
     clear_comp(M, w, t.lane, t.nl);
     team_sync(t.nl);
     float* wt = wtape ? wtape + (size_t)step * a.tape_step[it.group] : nullptr;
-    for (int k = 0; k < M.K; ++k) {
+    if (LANES) {
+      lane_from_scratch(M, w, lc, t.lane, ls);
+      const float tau0 = lc.act >= 0 ? lc.gear * w[M.o_ACT + lc.act] : 0.f;
+      for (int k = 0; k < M.K; ++k)
+        lane_substep(M, w, lc, ls, tau0, wt ? wt + (size_t)k * REC : nullptr, t.lane, t.nl, nm);
+      lane_to_scratch(M, w, lc, t.lane, ls);
+      team_sync(t.nl);
+    }
+    for (int k = 0; !LANES && k < M.K; ++k) {
       substep_dynamics(M, w, t.lane, t.nl, nm);
       if (wt) {   // keep the substep record for the adjoint
         record_save(wt + (size_t)k * REC, w, REC, t.lane, t.nl);
@@ -141,12 +158,8 @@ __device__ __forceinline__ void forward_item(const BatchedArgs& a, const DevMode
 // flight together, then wait for this lane's copies (the caller's team barrier
 // makes them visible to the team).
 __device__ __forceinline__ void record_load(const SMem& w, const float* src, int n, int lane, int nl) {
-  for (int j = lane; j < n / 4; j += nl) {
-    const unsigned dst = (unsigned)__cvta_generic_to_shared(&w[4 * j]);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src + 4 * j) : "memory");
-  }
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  record_request(w, 0, src, n, lane, nl);
+  record_wait();
 }
 
 // One work item of the window adjoint (reverse over steps).  Each step's
@@ -155,12 +168,19 @@ __device__ __forceinline__ void record_load(const SMem& w, const float* src, int
 // the workspace and reloaded by the reverse pass.  With the window tape the
 // forward window already kept every record (and the post-step state), and the
 // recompute is skipped.
+template <bool LANES>
 __device__ __forceinline__ void adjoint_item(const BatchedArgs& a, const DevModel& M, const WorkItem& it,
                                              const SMem& w, const Team& t) {
   const int nm = SHAC_DENSE_ROWS(a.dense_nm[it.group]);
   const GroupIO& io = a.io.g[it.group];
   const int REC = M.rec_floats;
   float* tape = a.tape + a.tape_off[it.group] + (size_t)(it.env0 + t.team) * ((size_t)M.K * REC);
+  LaneConst lc;
+  LaneState ls;
+  if (LANES) {
+    lc = lane_const(M, t.lane);
+    if (M.nseg > 0) muscle_clear(M, w, t.lane, t.nl);
+  }
   team_load(w, M.o_QB, a.qT_bar + io.q_off, M.nq, io.N, t.env, t.lane, t.nl);
   team_load(w, M.o_QDB, a.qdT_bar + io.qd_off, M.nv, io.N, t.env, t.lane, t.nl);
   for (int step = a.h - 1; step >= 0; --step) {
@@ -183,7 +203,14 @@ __device__ __forceinline__ void adjoint_item(const BatchedArgs& a, const DevMode
       for (int j = t.lane; j < M.nq; j += t.nl) w[M.o_Q + j] = post[j];
       for (int j = t.lane; j < M.nv; j += t.nl) w[M.o_QD + j] = post[M.nq + j];
       team_sync(t.nl);
-    } else {                    // recomputed once from the checkpoint
+    } else if (LANES) {         // recomputed once from the checkpoint
+      lane_from_scratch(M, w, lc, t.lane, ls);
+      const float tau0 = lc.act >= 0 ? lc.gear * w[M.o_ACT + lc.act] : 0.f;
+      for (int k = 0; k < M.K; ++k)
+        lane_substep(M, w, lc, ls, tau0, tape + (size_t)k * REC, t.lane, t.nl, nm);
+      lane_to_scratch(M, w, lc, t.lane, ls);
+      team_sync(t.nl);
+    } else {
       for (int k = 0; k < M.K; ++k) {
         substep_dynamics(M, w, t.lane, t.nl, nm);
         record_save(tape + (size_t)k * REC, w, REC, t.lane, t.nl);
@@ -193,7 +220,18 @@ __device__ __forceinline__ void adjoint_item(const BatchedArgs& a, const DevMode
     }
     if (t.lane == 0) reward_adjoint(M, w, a.reward_bar[(size_t)step * a.io.n_envs + io.env_off + t.env]);
     team_sync(t.nl);
-    for (int k = M.K - 1; k >= 0; --k) {
+    if (LANES) {
+      LaneBars g;
+      record_request(w, M.o_R, recs + (size_t)(M.K - 1) * REC, lane_record(M.L, M.nv, nm, M.root_free).items, t.lane, t.nl);
+      bars_from_scratch(M, w, lc, t.lane, g);
+      for (int k = M.K - 1; k >= 0; --k) {
+        const float* rec = recs + (size_t)k * REC;
+        lane_reverse(M, w, lc, g, rec, k > 0 ? rec - REC : nullptr, t.lane, t.nl, nm);
+      }
+      bars_to_scratch(M, w, lc, t.lane, g);
+      team_sync(t.nl);
+    }
+    for (int k = M.K - 1; !LANES && k >= 0; --k) {
       record_load(w, recs + (size_t)k * REC, REC, t.lane, t.nl);
       team_sync(t.nl);
       st_integrate_adj(M, w, t.lane, t.nl);
@@ -221,7 +259,7 @@ __device__ __forceinline__ void adjoint_item(const BatchedArgs& a, const DevMode
 // different arrays, so model fields are not reloaded after every scratch
 // store, and no call boundary splits the register allocation (measured on
 // the ant-like 2048-environment window: forward 5.99 -> 5.36 ms).
-template <bool ADJ>
+template <bool ADJ, bool LANES>
 __global__ void __maxnreg__(ADJ ? BATCHED_REGS_ADJOINT : BATCHED_REGS_FORWARD) k_batched(BatchedArgs a) {
   extern __shared__ __align__(16) float smem[];
   __shared__ DevModel s_models[MAX_GROUPS];
@@ -243,8 +281,8 @@ __global__ void __maxnreg__(ADJ ? BATCHED_REGS_ADJOINT : BATCHED_REGS_FORWARD) k
     Team t;
     setup_team(a, it, t);
     SMem w{wsm + (size_t)t.team * SHAC_ENV_STRIDE(a.env_stride[it.group])};
-    if (ADJ) adjoint_item(a, M, it, w, t);
-    else forward_item(a, M, it, w, t);
+    if (ADJ) adjoint_item<LANES>(a, M, it, w, t);
+    else forward_item<LANES>(a, M, it, w, t);
     __syncwarp();
   }
 }

@@ -27,6 +27,7 @@
 
 extern const char* const shac_jit_src_device;    // shac_device.cuh
 extern const char* const shac_jit_src_kernels;   // shac_kernels.cuh
+extern const char* const shac_jit_src_team;      // shac_team.cuh
 extern const char* const shac_jit_src_batched;   // shac_batched.cuh
 
 namespace shac {
@@ -49,7 +50,10 @@ const Field kFields[] = {
     {"o_LD", &DevModel::o_LD}, {"o_B", &DevModel::o_B}, {"o_T", &DevModel::o_T}, {"o_QDD", &DevModel::o_QDD},
     {"o_QC", &DevModel::o_QC}, {"o_QDC", &DevModel::o_QDC}, {"o_LAM", &DevModel::o_LAM},
     {"o_ITB", &DevModel::o_ITB}, {"o_SEGA", &DevModel::o_SEGA}, {"o_MW", &DevModel::o_MW},
-    {"o_RDB", &DevModel::o_RDB}, {"rec_floats", &DevModel::rec_floats}, {"env_floats", &DevModel::env_floats},
+    {"o_RDB", &DevModel::o_RDB}, {"o_X", &DevModel::o_X}, {"o_R", &DevModel::o_R},
+    {"o_MP", &DevModel::o_MP}, {"o_MB", &DevModel::o_MB}, {"o_MX", &DevModel::o_MX}, {"o_MF", &DevModel::o_MF},
+    {"mrows", &DevModel::mrows}, {"lanes_needed", &DevModel::lanes_needed},
+    {"nround", &DevModel::nround}, {"rec_floats", &DevModel::rec_floats}, {"env_floats", &DevModel::env_floats},
 };
 
 // Replace every `M.<field>` (as a whole word) by the field's value.
@@ -69,12 +73,19 @@ std::string parent_list(const std::vector<int>& parent) {
   return s;
 }
 
-std::string spec_string(int device, const DevModel& m, const std::vector<int>& parent, int lanes, int rows,
-                        int stride) {
+// the DOFs' ancestor masks ("1u,3u,...")
+std::string mask_list(const std::vector<int>& masks) {
+  std::string s;
+  for (size_t i = 0; i < masks.size(); ++i) s += (i ? "," : "") + std::to_string((unsigned)masks[i]) + "u";
+  return s;
+}
+
+std::string spec_string(int device, const DevModel& m, const std::vector<int>& parent, const std::vector<int>& masks,
+                        int lanes, int rows, int stride) {
   std::string s = "dev" + std::to_string(device) + ";lanes" + std::to_string(lanes) + ";rows" +
                   std::to_string(rows) + ";stride" + std::to_string(stride);
   for (const Field& f : kFields) s += ";" + std::string(f.name) + "=" + std::to_string(m.*(f.member));
-  return s + ";parents=" + parent_list(parent);
+  return s + ";parents=" + parent_list(parent) + ";masks=" + mask_list(masks);
 }
 
 // FNV-1a; 0 is reserved for the generic kernels
@@ -89,10 +100,10 @@ std::map<std::string, JitKernels> g_cache;
 
 }  // namespace
 
-shac_status jit_kernels(int device, const DevModel& m, const std::vector<int>& parent, int lanes, int rows,
-                        int stride, JitKernels* out, std::string* log) {
+shac_status jit_kernels(int device, const DevModel& m, const std::vector<int>& parent, const std::vector<int>& masks,
+                        int lanes, int rows, int stride, bool lane_form, JitKernels* out, std::string* log) {
   if ((int)parent.size() != m.L) return SHAC_ERR_INVALID_ARG;
-  const std::string spec = spec_string(device, m, parent, lanes, rows, stride);
+  const std::string spec = spec_string(device, m, parent, masks, lanes, rows, stride);
   std::lock_guard<std::mutex> lock(g_mutex);
   auto it = g_cache.find(spec);
   if (it != g_cache.end()) { *out = it->second; return SHAC_OK; }
@@ -104,17 +115,19 @@ shac_status jit_kernels(int device, const DevModel& m, const std::vector<int>& p
   const std::string h_device = with_literals(shac_jit_src_device, m);
   const std::string h_kernels = with_literals(shac_jit_src_kernels, m);
   const std::string h_batched = with_literals(shac_jit_src_batched, m);
-  const char* headers[] = {h_device.c_str(), h_kernels.c_str(), h_batched.c_str()};
-  const char* names[] = {"shac_device.cuh", "shac_kernels.cuh", "shac_batched.cuh"};
-  const char* main_src =
-      "#include \"shac_batched.cuh\"\n"
-      "template __global__ void shac::k_batched<false>(shac::BatchedArgs);\n"
-      "template __global__ void shac::k_batched<true>(shac::BatchedArgs);\n";
+  const std::string h_team = with_literals(shac_jit_src_team, m);
+  const char* headers[] = {h_device.c_str(), h_kernels.c_str(), h_team.c_str(), h_batched.c_str()};
+  const char* names[] = {"shac_device.cuh", "shac_kernels.cuh", "shac_team.cuh", "shac_batched.cuh"};
+  const char* fwd_name = lane_form ? "shac::k_batched<false, true>" : "shac::k_batched<false, false>";
+  const char* adj_name = lane_form ? "shac::k_batched<true, true>" : "shac::k_batched<true, false>";
+  std::string main_src = "#include \"shac_batched.cuh\"\n";
+  for (const char* k : {fwd_name, adj_name})
+    main_src += "template __global__ void " + std::string(k) + "(shac::BatchedArgs);\n";
   nvrtcProgram prog = nullptr;
-  if (nvrtcCreateProgram(&prog, main_src, "shac_batched_spec.cu", 3, headers, names) != NVRTC_SUCCESS)
+  if (nvrtcCreateProgram(&prog, main_src.c_str(), "shac_batched_spec.cu", 4, headers, names) != NVRTC_SUCCESS)
     return SHAC_ERR_CUDA;
-  nvrtcAddNameExpression(prog, "shac::k_batched<false>");
-  nvrtcAddNameExpression(prog, "shac::k_batched<true>");
+  nvrtcAddNameExpression(prog, fwd_name);
+  nvrtcAddNameExpression(prog, adj_name);
   const std::string arch = "--gpu-architecture=sm_" + std::to_string(major) + std::to_string(minor) + "a";
   char kbuf[64], lbuf[64], rbuf[64], sbuf[64];
   std::snprintf(kbuf, sizeof kbuf, "-DSHAC_SPEC_KEY=%uu", key);
@@ -122,7 +135,8 @@ shac_status jit_kernels(int device, const DevModel& m, const std::vector<int>& p
   std::snprintf(rbuf, sizeof rbuf, "-DSHAC_SPEC_ROWS=%d", rows);
   std::snprintf(sbuf, sizeof sbuf, "-DSHAC_SPEC_STRIDE=%d", stride);
   const std::string pdef = "-DSHAC_SPEC_PARENTS=" + parent_list(parent);
-  const char* opts[] = {arch.c_str(), "-std=c++17", "-lineinfo", kbuf, lbuf, rbuf, sbuf, pdef.c_str()};
+  const std::string adef = "-DSHAC_SPEC_ANC=" + mask_list(masks);
+  const char* opts[] = {arch.c_str(), "-std=c++17", "-lineinfo", kbuf, lbuf, rbuf, sbuf, pdef.c_str(), adef.c_str()};
   const nvrtcResult cr = nvrtcCompileProgram(prog, (int)(sizeof opts / sizeof opts[0]), opts);
   if (cr != NVRTC_SUCCESS) {
     if (log) {
@@ -137,8 +151,8 @@ shac_status jit_kernels(int device, const DevModel& m, const std::vector<int>& p
   }
   const char* lowered[2] = {nullptr, nullptr};
   size_t cubin_size = 0;
-  if (nvrtcGetLoweredName(prog, "shac::k_batched<false>", &lowered[0]) != NVRTC_SUCCESS ||
-      nvrtcGetLoweredName(prog, "shac::k_batched<true>", &lowered[1]) != NVRTC_SUCCESS ||
+  if (nvrtcGetLoweredName(prog, fwd_name, &lowered[0]) != NVRTC_SUCCESS ||
+      nvrtcGetLoweredName(prog, adj_name, &lowered[1]) != NVRTC_SUCCESS ||
       nvrtcGetCUBINSize(prog, &cubin_size) != NVRTC_SUCCESS || cubin_size == 0) {
     nvrtcDestroyProgram(&prog);
     return SHAC_ERR_CUDA;

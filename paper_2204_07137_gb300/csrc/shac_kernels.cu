@@ -163,23 +163,28 @@ void launch_plain_adj_store_state(const PlainGroup& g, float* qb, float* qdb, co
 
 namespace shac {
 
-#define k_batched_forward k_batched<false>
-#define k_batched_adjoint k_batched<true>
-
-void launch_batched_forward(const BatchedArgs& a, int grid, int block, size_t smem, cudaStream_t s) {
-  k_batched_forward<<<grid, block, smem, s>>>(a);
+template <bool ADJ>
+static const void* batched_kernel(bool lanes) {
+  return lanes ? (const void*)k_batched<ADJ, true> : (const void*)k_batched<ADJ, false>;
 }
-void launch_batched_adjoint(const BatchedArgs& a, int grid, int block, size_t smem, cudaStream_t s) {
-  k_batched_adjoint<<<grid, block, smem, s>>>(a);
+static void launch(const void* k, const BatchedArgs& a, int grid, int block, size_t smem, cudaStream_t s) {
+  void* args[] = {const_cast<BatchedArgs*>(&a)};
+  cudaLaunchKernel(k, dim3(grid), dim3(block), args, smem, s);
 }
-cudaError_t batched_set_smem_limit(size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(k_batched_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+void launch_batched_forward(const BatchedArgs& a, int grid, int block, size_t smem, bool lanes, cudaStream_t s) {
+  launch(batched_kernel<false>(lanes), a, grid, block, smem, s);
+}
+void launch_batched_adjoint(const BatchedArgs& a, int grid, int block, size_t smem, bool lanes, cudaStream_t s) {
+  launch(batched_kernel<true>(lanes), a, grid, block, smem, s);
+}
+cudaError_t batched_set_smem_limit(size_t smem, bool lanes) {
+  cudaError_t e = cudaFuncSetAttribute(batched_kernel<false>(lanes), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_batched_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return cudaFuncSetAttribute(batched_kernel<true>(lanes), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
-cudaError_t batched_occupancy(int* blocks_per_sm, int block, size_t smem, bool adjoint) {
-  if (adjoint) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_batched_adjoint, block, smem);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_batched_forward, block, smem);
+cudaError_t batched_occupancy(int* blocks_per_sm, int block, size_t smem, bool adjoint, bool lanes) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      blocks_per_sm, adjoint ? batched_kernel<true>(lanes) : batched_kernel<false>(lanes), block, smem);
 }
 
 }  // namespace shac

@@ -79,10 +79,11 @@ struct BatchedArgs {
 };
 
 #ifndef __CUDACC_RTC__
-void launch_batched_forward(const BatchedArgs& a, int grid, int block, size_t smem, cudaStream_t s);
-void launch_batched_adjoint(const BatchedArgs& a, int grid, int block, size_t smem, cudaStream_t s);
-cudaError_t batched_occupancy(int* blocks_per_sm, int block, size_t smem, bool adjoint);
-cudaError_t batched_set_smem_limit(size_t smem);
+// lanes: every group's team has a lane per link and DOF (the lane form's kernels)
+void launch_batched_forward(const BatchedArgs& a, int grid, int block, size_t smem, bool lanes, cudaStream_t s);
+void launch_batched_adjoint(const BatchedArgs& a, int grid, int block, size_t smem, bool lanes, cudaStream_t s);
+cudaError_t batched_occupancy(int* blocks_per_sm, int block, size_t smem, bool adjoint, bool lanes);
+cudaError_t batched_set_smem_limit(size_t smem, bool lanes);
 
 // Plain form: one environment per thread, one kernel per stage.
 struct PlainGroup {
