@@ -103,7 +103,10 @@ static void compute_muscle_slots(shac_model* m) {
   for (int i = 0; i < L; ++i) {
     m->ms_ptr[i] = s;
     const int n = m->lm_ptr[i + 1] - m->lm_ptr[i];
-    for (int k = 0; k < n; ++k) place[m->lm_idx[m->lm_ptr[i] + k]] = (k % m->mrows) * MSLOTS + s + k / m->mrows;
+    for (int k = 0; k < n; ++k) {
+      const int row = k % m->mrows;
+      place[m->lm_idx[m->lm_ptr[i] + k]] = row * MSLOTS + (s + k / m->mrows + row) % MSLOTS;
+    }
     s += (n + m->mrows - 1) / m->mrows;
   }
   m->ms_ptr[L] = s;
@@ -152,7 +155,6 @@ static void compute_lanes(shac_model* m) {
     const int l = lane_of[i];
     I(LI_LINK, l) = i; I(LI_JT, l) = m->jtype[i]; I(LI_Q, l) = m->qs[i];
     I(LI_C0, l) = m->lc_ptr[i]; I(LI_C1, l) = m->lc_ptr[i + 1];
-    I(LI_BASE, l) = m->parent[i] < 0;
     unsigned anc = 0;                     // the 2^r-th ancestors' lanes, 6 bits each (63: none)
     for (int r = 0; r < 5; ++r) {
       int j = i;
@@ -168,6 +170,13 @@ static void compute_lanes(shac_model* m) {
     for (int k = 0; k < 9; ++k) F(LF_JROT + k, l) = m->jrot[9 * i + k];
     for (int k = 0; k < 6; ++k) F(LF_ICOM + k, l) = m->icom[6 * i + k];
     F(LF_MASS, l) = m->mass[i];
+    if (m->lc_ptr[i] < m->lc_ptr[i + 1]) {   // its first contact sphere
+      const int e = m->lc_idx[m->lc_ptr[i]];
+      for (int k = 0; k < 3; ++k) F(LF_CPOS + k, l) = m->item_pos[3 * e + k];
+      F(LF_CRAD, l) = m->crad[e];
+    }
+    if (m->parent[i] < 0)
+      for (int k = 0; k < 3; ++k) F(LF_BASE + k, l) = -m->grav[k];
   }
   for (int d = 0; d < nv; ++d) {
     I(LI_DLINK, d) = m->dof_link[d];
@@ -205,6 +214,7 @@ static void compute_layout(shac_model* m) {
   d.lanes_needed = m->lanes_needed;
   d.nround = m->nround;
   d.mrows = m->mrows;
+  for (int i = 0; i < std::min(L, 32); ++i) d.par8[i] = (signed char)m->parent[i];
   take(d.o_B, nv); take(d.o_T, nv);
   take(d.o_LAM, nv); take(d.o_ITB, 10 * ni);
   take(d.o_SEGA, m->nseg);
@@ -479,13 +489,18 @@ static shac_status upload_model(const shac_model* m, Group& g) {
   return SHAC_OK;
 }
 
-static int default_lanes(const shac_model* m) {
+// Lanes per environment chosen for N environments: the fewest that give every
+// link and DOF a lane; below 16, where a component of the subtree sums ([Ic, F] has
+// 16) has no lane of its own, twice as many while the group's warps still fit the
+// GPU at once (8 an SM).  Cart-pole, 64 environments, us a step
+// forward + adjoint: two lanes 41 generic, 18 specialised; sixteen 26 and 15.
+static int default_lanes(const shac_model* m, int N, int num_sms) {
   const int par = std::max(m->nv, m->L);
-  if (par <= 2) return 2;
-  if (par <= 4) return 4;
-  if (par <= 8) return 8;
-  if (par <= 16) return 16;
-  return 32;
+  int lanes = 32;
+  for (int t : {16, 8, 4, 2})
+    if (par <= t) lanes = t;
+  while (lanes < 16 && (int64_t)N * 2 * lanes / 32 <= (int64_t)8 * num_sms) lanes *= 2;
+  return lanes;
 }
 
 // Register row capacity of the batched dense path: the smallest of the device
@@ -622,7 +637,7 @@ extern "C" shac_status shac_batch_create(const shac_model* const* models, const 
     Group g;
     g.m = models[gi];
     g.N = n_envs[gi];
-    g.lanes = default_lanes(g.m);
+    g.lanes = default_lanes(g.m, g.N, b->num_sms);
     shac_status st = upload_model(g.m, g);
     if (st != SHAC_OK) { shac_batch_destroy(b); return st; }
     GroupIO& io = b->io.g[gi];
@@ -685,7 +700,7 @@ extern "C" shac_status shac_batch_set_launch(shac_batch* b, int32_t group, int32
   if (warps < 0 || warps > 8) return SHAC_ERR_INVALID_ARG;
   for (int gi = 0; gi < (int)b->groups.size(); ++gi) {
     if (group >= 0 && gi != group) continue;
-    b->groups[gi].lanes = lanes == 0 ? default_lanes(b->groups[gi].m) : lanes;
+    b->groups[gi].lanes = lanes == 0 ? default_lanes(b->groups[gi].m, b->groups[gi].N, b->num_sms) : lanes;
   }
   if (warps > 0) b->warps_per_cta = warps;
   return build_items(b);

@@ -97,6 +97,7 @@ struct DevModel {
   // lane form (shac_team.cuh): lanes a team needs (DOFs, then the links without
   // one), doubling rounds, and the lane columns of the model's constants
   int lanes_needed, nround;
+  signed char par8[32];                  // link parents (models of at most 32 links)
   const int* ln_i;
   const float* ln_f;
   // lane form, muscles: the via-point items in MSLOTS columns of mrows (each

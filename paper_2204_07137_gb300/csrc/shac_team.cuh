@@ -28,20 +28,22 @@
 namespace shac {
 
 // This lane's share of the model (DevModel::ln_i, ln_f: one column per lane).
-enum { LI_LINK = 0, LI_JT, LI_ANC, LI_Q, LI_ACT, LI_C0, LI_C1, LI_DESC, LI_DLINK, LI_BASE, LI_N };
+enum { LI_LINK = 0, LI_JT, LI_ANC, LI_Q, LI_ACT, LI_C0, LI_C1, LI_DESC, LI_DLINK, LI_N };
 enum { LF_AXIS = 0, LF_JROT = 3, LF_JPOS = 12, LF_COM = 15, LF_ICOM = 18, LF_MASS = 24, LF_ARM, LF_DAMP, LF_GEAR,
-       LF_QLO, LF_QHI, LF_N };
+       LF_QLO, LF_QHI, LF_CPOS, LF_CRAD = LF_CPOS + 3, LF_BASE, LF_N = LF_BASE + 3 };
 constexpr int LANE_COLS = 32;
+constexpr float MIN_NORMAL = 1.17549435e-38f;
 constexpr int MSLOTS = 32;   // columns of the muscles' via-point items
 
 struct LaneConst {
   int link, jt, qi, act, c0, c1, dlink, ms0, ms1;
   unsigned anc, desc;
-  bool base, own;       // a root link (takes -g); lane < nv
-  V3 axis, jpos, com;
+  bool own;             // lane < nv
+  V3 axis, jpos, com, cpos, base;   // cpos, crad: the link's first contact; base: -g on a root link
   M33 jrot;
   float icom[6];
-  float mass, arm, damp, gear, qlo, qhi;
+  float mass, arm, damp, gear, qlo, qhi, crad;
+  float h, klim;
 };
 
 __device__ __forceinline__ LaneConst lane_const(const DevModel& M, int lane) {
@@ -52,7 +54,6 @@ __device__ __forceinline__ LaneConst lane_const(const DevModel& M, int lane) {
   LaneConst c;
   c.link = gi(LI_LINK); c.jt = gi(LI_JT); c.anc = (unsigned)gi(LI_ANC); c.qi = gi(LI_Q); c.act = gi(LI_ACT);
   c.c0 = gi(LI_C0); c.c1 = gi(LI_C1); c.desc = (unsigned)gi(LI_DESC); c.dlink = gi(LI_DLINK);
-  c.base = gi(LI_BASE) != 0;
   c.ms0 = c.ms1 = 0;
   if (M.nseg > 0 && c.link >= 0) { c.ms0 = __ldg(M.ms_ptr + c.link); c.ms1 = __ldg(M.ms_ptr + c.link + 1); }
   c.own = lane < M.nv;
@@ -65,6 +66,9 @@ __device__ __forceinline__ LaneConst lane_const(const DevModel& M, int lane) {
   for (int k = 0; k < 6; ++k) c.icom[k] = gf(LF_ICOM + k);
   c.mass = gf(LF_MASS); c.arm = gf(LF_ARM); c.damp = gf(LF_DAMP); c.gear = gf(LF_GEAR);
   c.qlo = gf(LF_QLO); c.qhi = gf(LF_QHI);
+  c.cpos = v3(gf(LF_CPOS), gf(LF_CPOS + 1), gf(LF_CPOS + 2)); c.crad = gf(LF_CRAD);
+  c.base = v3(gf(LF_BASE), gf(LF_BASE + 1), gf(LF_BASE + 2));
+  c.h = M.h; c.klim = M.klim;
   return c;
 }
 
@@ -90,6 +94,21 @@ __device__ __forceinline__ void path_sums(const DevModel& M, unsigned anc, int n
     const V3 pa = team_shfl(a, (int)(s & 31u), nl), pb = team_shfl(b, (int)(s & 31u), nl);
     if (s < 32u) { a = a + pa; b = b + pb; }
   }
+}
+
+// 1 / sqrt(x) to 2 ulp, a subnormal x taken as zero: rsqrtf without the scaling
+// that saves subnormal arguments, five instructions on the pivots' chain.
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// 1 / sqrt(x) for a normal x, refined by a Newton step of y -> y (3 - x y^2) / 2 to
+// within an ulp or so: what 1.f / sqrtf(x) gives, without its two special-case
+// branches, which keep the compiler from overlapping neighbouring evaluations.
+__device__ __forceinline__ float rsqrt_refined(float x) {
+  const float y = rsqrt_ftz(x);
+  return fmaf(0.5f * y, fmaf(-x * y, y, 1.f), y);
 }
 
 // 16-byte shared-memory accesses (o a multiple of 4).
@@ -150,36 +169,61 @@ __device__ __forceinline__ void record_request(const SMem& w, int o, const float
 }
 __device__ __forceinline__ void record_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// Subtree sums over blocks of `stride` floats per link (see subtree_sums).  The
-// generic loop carries the running sum of a chain (parent = i - 1) in a
-// register and reads the next link's value ahead; only a branch goes back to
-// memory.
+// Subtree sums of NC values a link; on return this lane's DOF's link's sums
+// (lanes from nv on: their link's or the first link's, not used).  Each link's
+// values go to its block of the exchange buffer, one component per lane adds
+// child to parent, last link first.  A specialised build does so at constant
+// addresses (150 cycles for the ant-like model's nine links and 16 components).
+// With the tree known at run time only, a chain's running sum (parent = i - 1)
+// stays in a register, the next link's value and parent are read ahead, and only
+// a branch goes back to memory.
 template <int NC>
-__device__ __forceinline__ void block_sums(const DevModel& M, const SMem& w, int o, int stride, int lane, int nl) {
-  for (int c = lane; c < NC; c += nl) {
+__device__ __forceinline__ void lane_sums(const DevModel& M, const SMem& w, float (&x)[NC], const LaneConst& c,
+                                          bool link, int lane, int nl) {
+  constexpr int N4 = (NC + 3) / 4;
+  if (link) {
+#pragma unroll
+    for (int j = 0; j < N4; ++j)
+      sts4(w, M.o_X + XB * c.link + 4 * j, x[4 * j], 4 * j + 1 < NC ? x[4 * j + 1 < NC ? 4 * j + 1 : 0] : 0.f,
+           4 * j + 2 < NC ? x[4 * j + 2 < NC ? 4 * j + 2 : 0] : 0.f, 4 * j + 3 < NC ? x[4 * j + 3 < NC ? 4 * j + 3 : 0] : 0.f);
+  }
+  team_sync(nl);
+  for (int k = lane; k < NC; k += nl) {
 #ifdef SHAC_SPEC_PARENTS
 #pragma unroll
     for (int i = M.L - 1; i > 0; --i) {
       const int p = link_parent(M, i);
-      if (p >= 0) w[o + stride * p + c] += w[o + stride * i + c];
+      if (p >= 0) w[M.o_X + XB * p + k] += w[M.o_X + XB * i + k];
     }
 #else
-    float x = w[o + stride * (M.L - 1) + c], carry = 0.f;
-    int p = M.L > 1 ? __ldg(M.parent + M.L - 1) : -1;
+    const int o = M.o_X + k;
+    int a = o + XB * (M.L - 1), p = M.par8[M.L - 1];
+    float v = w[a], carry = 0.f;
     for (int i = M.L - 1; i > 0; --i) {
-      const float xn = w[o + stride * (i - 1) + c];
-      const int pn = __ldg(M.parent + i - 1);
-      const float s = x + carry;
-      w[o + stride * i + c] = s;
-      carry = 0.f;
-      x = xn;
-      if (p == i - 1) carry = s;
-      else if (p >= 0) w[o + stride * p + c] += s;
+      const float vn = w[a - XB];
+      const int pn = M.par8[i - 1];
+      const float s = v + carry;
+      w[a] = s;
+      const bool chain = p == i - 1;
+      if (!chain && p >= 0) w[o + XB * p] += s;
+      carry = chain ? s : 0.f;
+      v = vn;
       p = pn;
+      a -= XB;
     }
-    w[o + c] = x + carry;
+    w[a] = v + carry;
 #endif
   }
+  team_sync(nl);
+#pragma unroll
+  for (int j = 0; j < N4; ++j) {
+    const float4 v = lds4(w, M.o_X + XB * c.dlink + 4 * j);
+    x[4 * j] = v.x;
+    if (4 * j + 1 < NC) x[4 * j + 1 < NC ? 4 * j + 1 : 0] = v.y;
+    if (4 * j + 2 < NC) x[4 * j + 2 < NC ? 4 * j + 2 : 0] = v.z;
+    if (4 * j + 3 < NC) x[4 * j + 3 < NC ? 4 * j + 3 : 0] = v.w;
+  }
+  team_sync(nl);   // the blocks are free again
 }
 
 // Which entries of the factor exist, and which DOFs may be eliminated
@@ -220,7 +264,7 @@ struct Dense {
   template <int LV, int K>
   static __device__ __forceinline__ void pivot(float diag, float (&inv)[NM], float b, float (&y)[NM], int nl) {
     if constexpr (dof_level(K) == LV) {
-      inv[K] = rsqrtf(team_shfl(diag, K, nl));
+      inv[K] = rsqrt_ftz(team_shfl(diag, K, nl));
       y[K] = team_shfl(b, K, nl) * inv[K];
     }
   }
@@ -289,22 +333,37 @@ struct Dense {
   // Assemble, factor and solve (M + diag(arm)) x = b; returns x of this lane's
   // DOF and 1 / L_kk in idiag.  sw, sv: the lane's motion subspace; the vectors
   // Ic_b S_b of every DOF are at of.
-  template <int... B>
-  static __device__ __forceinline__ void assemble(const SMem& w, int of, V3 sw, V3 sv, const LaneConst& c, int lane,
-                                                  float (&row)[NM], float& diag, iseq<B...>) {
+  // The columns go in groups whose vectors are all read before the first product
+  // (one at a time, every column waited for its own reads: 54 cycles each).
+  static constexpr int GROUP = 7;
+  template <int B0, int... B>
+  static __device__ __forceinline__ void assemble_group(const SMem& w, int of, V3 sw, V3 sv, const LaneConst& c,
+                                                        int lane, float (&row)[NM], float& diag, iseq<B...>) {
+    float4 f0[sizeof...(B)];
+    float2 f1[sizeof...(B)];
     ([&] {
-      const float4 f0 = lds4(w, of + XF * B);
-      const float2 f1 = *reinterpret_cast<const float2*>(&w[of + XF * B + 4]);
-      const float p = dot(sw, v3(f0.x, f0.y, f0.z)) + dot(sv, v3(f0.w, f1.x, f1.y));
-      float v = ((c.desc >> B) & 1u) ? p : 0.f;
-      if (B == lane) { v += c.arm; diag = v; }
-      row[B] = v;
+      f0[B] = lds4(w, of + XF * (B0 + B));
+      f1[B] = *reinterpret_cast<const float2*>(&w[of + XF * (B0 + B) + 4]);
     }(), ...);
+    ([&] {
+      const float p = dot(sw, v3(f0[B].x, f0[B].y, f0[B].z)) + dot(sv, v3(f0[B].w, f1[B].x, f1[B].y));
+      float v = ((c.desc >> (B0 + B)) & 1u) ? p : 0.f;
+      if (B0 + B == lane) { v += c.arm; diag = v; }
+      row[B0 + B] = v;
+    }(), ...);
+  }
+  template <int B0 = 0>
+  static __device__ __forceinline__ void assemble(const SMem& w, int of, V3 sw, V3 sv, const LaneConst& c, int lane,
+                                                  float (&row)[NM], float& diag) {
+    if constexpr (B0 < NM) {
+      assemble_group<B0>(w, of, sw, sv, c, lane, row, diag, make_iseq<(NM - B0 < GROUP ? NM - B0 : GROUP)>{});
+      assemble<B0 + GROUP>(w, of, sw, sv, c, lane, row, diag);
+    }
   }
   static __device__ __forceinline__ float solve(const SMem& w, float* fac, int rs, int of, int ol, V3 sw, V3 sv,
                                                 float b, const LaneConst& c, int lane, int nl, float& idiag) {
     float row[NM], diag = 1.f;
-    assemble(w, of, sw, sv, c, lane, row, diag, make_iseq<NM>{});
+    assemble(w, of, sw, sv, c, lane, row, diag);
     factor(w, ol, row, diag, idiag, b, lane, nl, make_iseq<NM>{});
     team_sync(nl);
     float ls[NM];
@@ -410,23 +469,30 @@ __device__ __forceinline__ void lane_local(const DevModel& M, const SMem& w, con
   k.si[6] = Iw.m[8] + m * (cc - cm.z * cm.z); k.si[7] = Iw.m[1] - m * cm.x * cm.y;
   k.si[8] = Iw.m[2] - m * cm.x * cm.z; k.si[9] = Iw.m[5] - m * cm.y * cm.z;
   k.wn = k.wf = v3(0.f, 0.f, 0.f);
-  for (int e = c.c0; e < c.c1; ++e) {   // contact spheres (the model of lk_local)
-    const int ci = __ldg(M.lc_idx + e);
-    V3 x = k.P + mul(k.R, cld3(M.item_pos + 3 * ci));
-    x.z -= __ldg(M.crad + ci);
+  V3 xl = c.cpos;
+  float rad = c.crad;
+  for (int e = c.c0; e < c.c1;) {   // contact spheres (the model of lk_local)
+    V3 x = k.P + mul(k.R, xl);
+    x.z -= rad;
     const float d = x.z + zroot;
     V3 f = v3(0.f, 0.f, 0.f);
     if (d < 0.f) {
       const V3 vp = k.Vv + cross(k.Vw, x);
       const float fn = (-M.ke + M.kd * vp.z) * d;
-      const float vt = sqrtf(vp.x * vp.x + vp.y * vp.y);
-      const float afn = fabsf(fn);
-      if (M.kt * vt <= M.mu * afn) { f.x = -M.kt * vp.x; f.y = -M.kt * vp.y; }
-      else { const float sc = M.mu * afn / vt; f.x = -sc * vp.x; f.y = -sc * vp.y; }
+      const float v2 = vp.x * vp.x + vp.y * vp.y;
+      const float iv = v2 > MIN_NORMAL ? rsqrt_refined(v2) : 0.f;   // 1 / |v_t|
+      const float fmax = M.mu * fabsf(fn);
+      const float sc = M.kt * (v2 * iv) <= fmax ? M.kt : fmax * iv;
+      f.x = -sc * vp.x; f.y = -sc * vp.y;
       f.z = fn;
     }
     k.wn = k.wn + cross(x, f);
     k.wf = k.wf + f;
+    if (++e < c.c1) {
+      const int ci = __ldg(M.lc_idx + e);
+      xl = cld3(M.item_pos + 3 * ci);
+      rad = __ldg(M.crad + ci);
+    }
   }
   V3 bn, bf;
   si_mul(k.si, k.aw, k.av, k.fn, k.ff);
@@ -435,8 +501,15 @@ __device__ __forceinline__ void lane_local(const DevModel& M, const SMem& w, con
   k.ff = k.ff + cross(k.Vw, bf) - k.wf;
 }
 
+// Segments a lane takes together: all their reads come before the first store
+// (which could alias them for all the compiler knows), so their latencies overlap.
+constexpr int SEG_GROUP = 2;
+
 // Muscles of the lane form.  The via-point items are laid out in MSLOTS columns
-// of mrows (item j of column s at j * MSLOTS + s), every column one link's items
+// of mrows (row j of column s at j * MSLOTS + (s + j) % MSLOTS: both a row and
+// the consecutive items of a link, which neighbouring lanes write, lie on
+// different banks; without the shift a segment step took 770 cycles, with it
+// 580), every column one link's items
 // and every link at least its share of columns, so that the per-link sums take
 // mrows conflict-free steps whatever the distribution of the items over the
 // links (a lane per link takes as many steps as the busiest link has items: 99
@@ -478,32 +551,42 @@ __device__ __forceinline__ void plane_st(const SMem& w, int o, int n, int i, V3 
 }
 __device__ __forceinline__ void muscle_forward(const DevModel& M, const SMem& w, int lane, int nl) {
   const int n = MSLOTS * M.mrows;
-#pragma unroll 2
-  for (int sg = lane; sg < M.nseg; sg += nl) {   // seg_forward
-    const Segment s = muscle_segment(M, sg);
-    auto point = [&](int link, V3 p) {
-      const int o = M.o_MP + 12 * link;
-      const float4 a = lds4(w, o), b = lds4(w, o + 4), c = lds4(w, o + 8);
-      M33 R;
-      R.m[0] = a.x; R.m[1] = a.y; R.m[2] = a.z; R.m[3] = a.w; R.m[4] = b.x; R.m[5] = b.y; R.m[6] = b.z; R.m[7] = b.w;
-      R.m[8] = c.x;
-      return v3(c.y, c.z, c.w) + mul(R, p);
-    };
-    const V3 x0 = point(s.l0, s.p0), x1 = point(s.l1, s.p1);
-    const float a = fminf(fmaxf(w[M.o_ACT + M.ntact + s.mus], 0.f), 1.f);
-    const V3 dv = x1 - x0;
-    const V3 f = (a * s.fmax) * ((1.f / sqrtf(dot(dv, dv))) * dv);
-    plane_st(w, M.o_MX, n, s.i0, x0);
-    plane_st(w, M.o_MX, n, s.i1, x1);
-    plane_st(w, M.o_MF, n, s.i0, f);
-    plane_st(w, M.o_MF, n, s.i1, -f);
+  auto point = [&](int link, V3 p) {
+    const int o = M.o_MP + 12 * link;
+    const float4 a = lds4(w, o), b = lds4(w, o + 4), c = lds4(w, o + 8);
+    M33 R;
+    R.m[0] = a.x; R.m[1] = a.y; R.m[2] = a.z; R.m[3] = a.w; R.m[4] = b.x; R.m[5] = b.y; R.m[6] = b.z; R.m[7] = b.w;
+    R.m[8] = c.x;
+    return v3(c.y, c.z, c.w) + mul(R, p);
+  };
+  for (int s0 = lane; s0 < M.nseg; s0 += SEG_GROUP * nl) {   // seg_forward
+    V3 x0[SEG_GROUP], x1[SEG_GROUP], f[SEG_GROUP];
+    int i0[SEG_GROUP], i1[SEG_GROUP];
+#pragma unroll
+    for (int g = 0; g < SEG_GROUP; ++g) {
+      const Segment s = muscle_segment(M, min(s0 + g * nl, M.nseg - 1));
+      x0[g] = point(s.l0, s.p0); x1[g] = point(s.l1, s.p1);
+      i0[g] = s.i0; i1[g] = s.i1;
+      const float a = fminf(fmaxf(w[M.o_ACT + M.ntact + s.mus], 0.f), 1.f);
+      const V3 dv = x1[g] - x0[g];
+      f[g] = (a * s.fmax) * (rsqrt_refined(dot(dv, dv)) * dv);
+    }
+#pragma unroll
+    for (int g = 0; g < SEG_GROUP; ++g) {
+      if (s0 + g * nl < M.nseg) {
+        plane_st(w, M.o_MX, n, i0[g], x0[g]);
+        plane_st(w, M.o_MX, n, i1[g], x1[g]);
+        plane_st(w, M.o_MF, n, i0[g], f[g]);
+        plane_st(w, M.o_MF, n, i1[g], -f[g]);
+      }
+    }
   }
   team_sync(nl);
   for (int c = lane; c < MSLOTS; c += nl) {
     V3 wn = v3(0.f, 0.f, 0.f), wf = wn;
 #pragma unroll 4
     for (int j = 0; j < M.mrows; ++j) {
-      const V3 x = plane_ld(w, M.o_MX, n, MSLOTS * j + c), f = plane_ld(w, M.o_MF, n, MSLOTS * j + c);
+      const V3 x = plane_ld(w, M.o_MX, n, MSLOTS * j + ((c + j) & (MSLOTS - 1))), f = plane_ld(w, M.o_MF, n, MSLOTS * j + ((c + j) & (MSLOTS - 1)));
       wn = wn + cross(x, f);
       wf = wf + f;
     }
@@ -517,23 +600,37 @@ __device__ __forceinline__ void muscle_forward(const DevModel& M, const SMem& w,
 // cotangents x_bar and of x_bar x^T.
 __device__ __forceinline__ void muscle_reverse(const DevModel& M, const SMem& w, int lane, int nl) {
   const int n = MSLOTS * M.mrows;
-#pragma unroll 2
-  for (int sg = lane; sg < M.nseg; sg += nl) {
-    const Segment s = muscle_segment(M, sg);
-    const V3 x0 = plane_ld(w, M.o_MX, n, s.i0), x1 = plane_ld(w, M.o_MX, n, s.i1);
-    const V3 n0 = ld3(w, M.o_MB + 6 * s.l0), e0 = ld3(w, M.o_MB + 6 * s.l0 + 3);
-    const V3 n1 = ld3(w, M.o_MB + 6 * s.l1), e1 = ld3(w, M.o_MB + 6 * s.l1 + 3);
-    const float araw = w[M.o_ACT + M.ntact + s.mus];
-    const float F = fminf(fmaxf(araw, 0.f), 1.f) * s.fmax;
-    const V3 dv = x1 - x0;
-    const float il = 1.f / sqrtf(dot(dv, dv));
-    const V3 u = il * dv, f = F * u;
-    const V3 g = (cross(x0, n0) - e0) - (cross(x1, n1) - e1);   // f0_bar - f1_bar
-    const V3 ub = F * g;
-    const V3 dvb = il * (ub - dot(u, ub) * u);
-    plane_st(w, M.o_MF, n, s.i0, cross(n0, f) - dvb);
-    plane_st(w, M.o_MF, n, s.i1, dvb - cross(n1, f));
-    w[M.o_SEGA + sg] = (araw > 0.f && araw < 1.f) ? dot(u, g) * s.fmax : 0.f;
+  for (int s0 = lane; s0 < M.nseg; s0 += SEG_GROUP * nl) {
+    V3 b0[SEG_GROUP], b1[SEG_GROUP];
+    float ab[SEG_GROUP];
+    int i0[SEG_GROUP], i1[SEG_GROUP];
+#pragma unroll
+    for (int k = 0; k < SEG_GROUP; ++k) {
+      const Segment s = muscle_segment(M, min(s0 + k * nl, M.nseg - 1));
+      const V3 x0 = plane_ld(w, M.o_MX, n, s.i0), x1 = plane_ld(w, M.o_MX, n, s.i1);
+      const V3 n0 = ld3(w, M.o_MB + 6 * s.l0), e0 = ld3(w, M.o_MB + 6 * s.l0 + 3);
+      const V3 n1 = ld3(w, M.o_MB + 6 * s.l1), e1 = ld3(w, M.o_MB + 6 * s.l1 + 3);
+      i0[k] = s.i0; i1[k] = s.i1;
+      const float araw = w[M.o_ACT + M.ntact + s.mus];
+      const float F = fminf(fmaxf(araw, 0.f), 1.f) * s.fmax;
+      const V3 dv = x1 - x0;
+      const float il = rsqrt_refined(dot(dv, dv));
+      const V3 u = il * dv, f = F * u;
+      const V3 g = (cross(x0, n0) - e0) - (cross(x1, n1) - e1);   // f0_bar - f1_bar
+      const V3 ub = F * g;
+      const V3 dvb = il * (ub - dot(u, ub) * u);
+      b0[k] = cross(n0, f) - dvb;
+      b1[k] = dvb - cross(n1, f);
+      ab[k] = (araw > 0.f && araw < 1.f) ? dot(u, g) * s.fmax : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < SEG_GROUP; ++k) {
+      if (s0 + k * nl < M.nseg) {
+        plane_st(w, M.o_MF, n, i0[k], b0[k]);
+        plane_st(w, M.o_MF, n, i1[k], b1[k]);
+        w[M.o_SEGA + s0 + k * nl] = ab[k];
+      }
+    }
   }
   team_sync(nl);
   for (int mu = lane; mu < M.nm; mu += nl) {
@@ -548,7 +645,7 @@ __device__ __forceinline__ void muscle_reverse(const DevModel& M, const SMem& w,
     for (int j = 0; j < 9; ++j) Q.m[j] = 0.f;
 #pragma unroll 4
     for (int j = 0; j < M.mrows; ++j) {
-      const V3 x = plane_ld(w, M.o_MX, n, MSLOTS * j + c), xb = plane_ld(w, M.o_MF, n, MSLOTS * j + c);
+      const V3 x = plane_ld(w, M.o_MX, n, MSLOTS * j + ((c + j) & (MSLOTS - 1))), xb = plane_ld(w, M.o_MF, n, MSLOTS * j + ((c + j) & (MSLOTS - 1)));
       Pb = Pb + xb;
       add_outer(Q, xb, x);
     }
@@ -605,7 +702,7 @@ __device__ __forceinline__ void lane_substep(const DevModel& M, const SMem& w, c
   path_sums(M, c.anc, nl, k.Vw, k.Vv);
   k.aw = cross(k.Vw, uw);
   k.av = cross(k.Vw, uv) + cross(k.Vv, uw);
-  if (c.base) k.av = k.av + v3(-M.grav[0], -M.grav[1], -M.grav[2]);
+  k.av = k.av + c.base;
   path_sums(M, c.anc, nl, k.aw, k.av);
   V3 sw = c.jt == J_REV ? ax : v3(0.f, 0.f, 0.f);
   V3 sv = c.jt == J_REV ? cross(k.P, ax) : (c.jt == J_PRIS ? ax : v3(0.f, 0.f, 0.f));
@@ -650,24 +747,18 @@ __device__ __forceinline__ void lane_substep(const DevModel& M, const SMem& w, c
     stg4(r + 7 * fs, k.wn.x, k.wn.y, k.wn.z, k.wf.x);
     *reinterpret_cast<float2*>(rec + ro.fx + 2 * c.link) = make_float2(k.wf.y, k.wf.z);
   }
-  // composite inertias and total forces
-  const int ox = M.o_X, of = M.o_X + XB * M.L;
-  if (link) {
-    const int o = ox + XB * c.link;
-    sts4(w, o, k.si[0], k.si[1], k.si[2], k.si[3]);
-    sts4(w, o + 4, k.si[4], k.si[5], k.si[6], k.si[7]);
-    sts4(w, o + 8, k.si[8], k.si[9], k.fn.x, k.fn.y);
-    sts4(w, o + 12, k.fn.z, k.ff.x, k.ff.y, k.ff.z);
-  }
-  team_sync(nl);
-  block_sums<16>(M, w, ox, XB, lane, nl);
-  team_sync(nl);
+  // composite inertias and total forces of this lane's DOF's link
+  const int of = M.o_X + XB * M.L;
+  float x[16];
+#pragma unroll
+  for (int j = 0; j < 10; ++j) x[j] = k.si[j];
+  x[10] = k.fn.x; x[11] = k.fn.y; x[12] = k.fn.z;
+  x[13] = k.ff.x; x[14] = k.ff.y; x[15] = k.ff.z;
+  lane_sums(M, w, x, c, link, lane, nl);
   // right-hand side and the vectors Ic S
   float b = 0.f;
   {
-    const int o = ox + XB * c.dlink;
-    const float4 a0 = lds4(w, o), a1 = lds4(w, o + 4), a2 = lds4(w, o + 8), a3 = lds4(w, o + 12);
-    const float ic[10] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w, a2.x, a2.y};
+    const float ic[10] = {x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7], x[8], x[9]};
     V3 fn, ff;
     si_mul(ic, sw, sv, fn, ff);
     if (lane < nm) {
@@ -677,10 +768,10 @@ __device__ __forceinline__ void lane_substep(const DevModel& M, const SMem& w, c
     if (c.own) {
       float t = tau0;
       if (c.jt == J_REV || c.jt == J_PRIS) {
-        if (s.q < c.qlo) t += M.klim * (c.qlo - s.q);
-        else if (s.q > c.qhi) t += M.klim * (c.qhi - s.q);
+        if (s.q < c.qlo) t += c.klim * (c.qlo - s.q);
+        else if (s.q > c.qhi) t += c.klim * (c.qhi - s.q);
       }
-      b = t - c.damp * s.qd - (dot(sw, v3(a2.z, a2.w, a3.x)) + dot(sv, v3(a3.y, a3.z, a3.w)));
+      b = t - c.damp * s.qd - (dot(sw, v3(x[10], x[11], x[12])) + dot(sv, v3(x[13], x[14], x[15])));
     }
   }
   team_sync(nl);
@@ -826,7 +917,7 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
     const float hh = 0.5f * h;
     const V3 nu = u + hh * (rw * om1 + cross(u, om1));
     const float nw = rw - hh * dot(u, om1);
-    const float inv = 1.f / sqrtf(dot(nu, nu) + nw * nw);
+    const float inv = rsqrt_refined(dot(nu, nu) + nw * nw);
     const V3 qu1 = inv * nu;
     const float qw1 = inv * nw;
     const V3 qub = v3(g.rqb[3], g.rqb[4], g.rqb[5]);
@@ -874,12 +965,12 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
   }
   k.aw = k.aw + cross(k.Vw, uw);
   k.av = k.av + cross(k.Vw, uv) + cross(k.Vv, uw);
-  if (c.base) k.av = k.av + v3(-M.grav[0], -M.grav[1], -M.grav[2]);
+  k.av = k.av + c.base;
   path_sums2(M, c.anc, nl, k.aw, k.av, nb, fb);
   // the joint forces of this lane's DOF (dof_adj_force)
   if (c.own) {
     g.actb += lam * c.gear;
-    if (one && (q < c.qlo || q > c.qhi)) g.qb -= lam * M.klim;
+    if (one && (q < c.qlo || q > c.qhi)) g.qb -= lam * c.klim;
     g.qdb -= lam * c.damp;
   }
   // local force and its reverse (lk_adj_local)
@@ -889,15 +980,11 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
   k.fn = k.fn + cross(k.Vw, bn) + cross(k.Vv, bf) - k.wn;
   k.ff = k.ff + cross(k.Vw, bf) - k.wf;
   si_mul(k.si, nb, fb, abn, abf);
-  const int ox = M.o_X;
-  if (link) {
-    const int o = ox + XB * c.link;
-    sts4(w, o, k.fn.x, k.fn.y, k.fn.z, k.ff.x);
-    sts4(w, o + 4, k.ff.y, k.ff.z, abn.x, abn.y);
-    sts4(w, o + 8, abn.z, abf.x, abf.y, abf.z);
-  }
-  team_sync(nl);
-  block_sums<12>(M, w, ox, XB, lane, nl);
+  // total forces and A_bar
+  float xs[12] = {k.fn.x, k.fn.y, k.fn.z, k.ff.x, k.ff.y, k.ff.z, abn.x, abn.y, abn.z, abf.x, abf.y, abf.z};
+  lane_sums(M, w, xs, c, link, lane, nl);
+  const V3 Fn = v3(xs[0], xs[1], xs[2]), Ff = v3(xs[3], xs[4], xs[5]);
+  const V3 an = v3(xs[6], xs[7], xs[8]), af = v3(xs[9], xs[10], xs[11]);
   V3 hb = v3(0.f, 0.f, 0.f);
   M33 G;
 #pragma unroll
@@ -931,36 +1018,34 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
     add_outer(Rb, Pb, c.com);
   }
   float depth = 0.f;   // cotangent of the root height through the contact depths
-  for (int e = c.c0; e < c.c1; ++e) {
-    const int ci = __ldg(M.lc_idx + e);
-    const V3 xl = cld3(M.item_pos + 3 * ci);
+  V3 xl = c.cpos;
+  float rad = c.crad;
+  for (int e = c.c0; e < c.c1;) {
     V3 x = k.P + mul(k.R, xl);
-    x.z -= __ldg(M.crad + ci);
+    x.z -= rad;
     const float dep = x.z + zroot;
     if (dep < 0.f) {
       const V3 vp = k.Vv + cross(k.Vw, x);
       const float fn = (-M.ke + M.kd * vp.z) * dep;
-      const float vt = sqrtf(vp.x * vp.x + vp.y * vp.y);
-      const float afn = fabsf(fn);
+      const float v2 = vp.x * vp.x + vp.y * vp.y;
+      const float iv = v2 > MIN_NORMAL ? rsqrt_refined(v2) : 0.f;   // 1 / |v_t|
+      const float fmax = M.mu * fabsf(fn);
       const V3 neb = -nb;
       const V3 fbar = cross(neb, x) - fb;
       float fnb = fbar.z;
       V3 f, vpb = v3(0.f, 0.f, 0.f);
       f.z = fn;
-      if (M.kt * vt <= M.mu * afn) {
-        f.x = -M.kt * vp.x; f.y = -M.kt * vp.y;
-        vpb.x = -M.kt * fbar.x;
-        vpb.y = -M.kt * fbar.y;
-      } else {
-        const float sc = M.mu * afn / vt;
-        f.x = -sc * vp.x; f.y = -sc * vp.y;
-        const float sb = -(fbar.x * vp.x + fbar.y * vp.y);
-        vpb.x = -sc * fbar.x;
-        vpb.y = -sc * fbar.y;
-        fnb += sb * M.mu * (fn >= 0.f ? 1.f : -1.f) / vt;
-        const float vtb = -sb * sc / vt;
-        vpb.x += vtb * vp.x / vt;
-        vpb.y += vtb * vp.y / vt;
+      const bool slow = M.kt * (v2 * iv) <= fmax;
+      const float sc = slow ? M.kt : fmax * iv;
+      f.x = -sc * vp.x; f.y = -sc * vp.y;
+      vpb.x = -sc * fbar.x;
+      vpb.y = -sc * fbar.y;
+      if (!slow) {
+        const float sb = -(fbar.x * vp.x + fbar.y * vp.y) * iv;
+        fnb += sb * (fn >= 0.f ? M.mu : -M.mu);
+        const float vtb = -sb * sc * iv;
+        vpb.x += vtb * vp.x;
+        vpb.y += vtb * vp.y;
       }
       V3 xb = cross(f, neb);
       const float db = fnb * (-M.ke + M.kd * vp.z);   // fn = (-ke + kd ddot) d, d = x.z + root height
@@ -972,6 +1057,11 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
       xb = xb + cross(vpb, k.Vw);
       Pb = Pb + xb;
       add_outer(Rb, xb, xl);
+    }
+    if (++e < c.c1) {
+      const int ci = __ldg(M.lc_idx + e);
+      xl = cld3(M.item_pos + 3 * ci);
+      rad = __ldg(M.crad + ci);
     }
   }
   V3 Pm = v3(0.f, 0.f, 0.f);   // muscles: their points' cotangents and moments sum x_bar x^T
@@ -996,32 +1086,14 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
       }
     }
   }
-  // total forces and A_bar; V_bar's own term with A_bar, and its sums
-  team_sync(nl);
-  V3 Fn, Ff, an, af, Fn0, Ff0, an0, af0;
-  auto read12 = [&](int o, V3& p, V3& q_, V3& r, V3& s) {
-    const float4 a0 = lds4(w, o), a1 = lds4(w, o + 4), a2 = lds4(w, o + 8);
-    p = v3(a0.x, a0.y, a0.z); q_ = v3(a0.w, a1.x, a1.y); r = v3(a1.z, a1.w, a2.x); s = v3(a2.y, a2.z, a2.w);
-  };
-  const int oi = ox + XB * (link ? c.link : 0);
-  read12(oi, Fn, Ff, an, af);
-  if (M.root_free) read12(ox, Fn0, Ff0, an0, af0);
+  // V_bar's own term with A_bar, and its sums
   vwb = vwb + cross(uw, an) + cross(uv, af);
   vvb = vvb + cross(uw, af);
-  const int ov = ox + XB * M.L;   // the V_bar blocks (8 floats per link) beside the first ones
-  if (link) {
-    sts4(w, ov + XF * c.link, vwb.x, vwb.y, vwb.z, vvb.x);
-    *reinterpret_cast<float2*>(&w[ov + XF * c.link + 4]) = make_float2(vvb.y, vvb.z);
+  {
+    float xv[6] = {vwb.x, vwb.y, vwb.z, vvb.x, vvb.y, vvb.z};
+    lane_sums(M, w, xv, c, link, lane, nl);
+    vwb = v3(xv[0], xv[1], xv[2]); vvb = v3(xv[3], xv[4], xv[5]);
   }
-  team_sync(nl);
-  block_sums<6>(M, w, ov, XF, lane, nl);
-  team_sync(nl);
-  auto read6 = [&](int o, V3& p, V3& q_) {
-    const float4 a0 = lds4(w, o);
-    const float2 a1 = *reinterpret_cast<const float2*>(&w[o + 4]);
-    p = v3(a0.x, a0.y, a0.z); q_ = v3(a0.w, a1.x, a1.y);
-  };
-  read6(ov + XF * (link ? c.link : 0), vwb, vvb);
   // one-DOF joint terms and the moment Q of this link's own pose cotangents
   if (one) {
     const V3 tw = cross(an, k.Vw) + cross(af, k.Vv) + vwb, tv = cross(af, k.Vw) + vvb;
@@ -1043,46 +1115,35 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
 #pragma unroll
     for (int j = 0; j < 9; ++j) Q.m[j] += Qm.m[j];
   }
-  if (link) {   // the first blocks' readers are past the V_bar barriers
-    sts4(w, oi, Q.m[0], Q.m[1], Q.m[2], Q.m[3]);
-    sts4(w, oi + 4, Q.m[4], Q.m[5], Q.m[6], Q.m[7]);
-    sts4(w, oi + 8, Q.m[8], Pb.x, Pb.y, Pb.z);
-    w[oi + 12] = depth;
-  }
-  team_sync(nl);
-  block_sums<13>(M, w, ox, XB, lane, nl);
-  team_sync(nl);
+  float xq[13] = {Q.m[0], Q.m[1], Q.m[2], Q.m[3], Q.m[4], Q.m[5], Q.m[6], Q.m[7], Q.m[8], Pb.x, Pb.y, Pb.z, depth};
+  lane_sums(M, w, xq, c, link, lane, nl);
   // q_bar: a revolute joint's is a . (axial(Q) - P x P_bar), a prismatic one's a . P_bar
   if (one) {
-    const float4 a0 = lds4(w, oi), a1 = lds4(w, oi + 4), a2 = lds4(w, oi + 8);
-    const V3 axial = v3(a1.w - a1.y, a0.z - a1.z, a0.w - a0.y), pb = v3(a2.y, a2.z, a2.w);
+    const V3 axial = v3(xq[7] - xq[5], xq[2] - xq[6], xq[3] - xq[1]), pb = v3(xq[9], xq[10], xq[11]);
     g.qb += c.jt == J_REV ? dot(ax, axial - cross(k.P, pb)) : dot(ax, pb);
   }
-  if (M.root_free) {   // the root's six DOFs and its quaternion, on every lane
-    V3 vw0, vv0;
-    read6(ov, vw0, vv0);
+  if (M.root_free) {   // the root's six DOFs and its quaternion: lanes 0 to 5 hold the root's sums, the others' values
+                       // are not used
     const V3 w3 = v3(rqd[0], rqd[1], rqd[2]), v3_ = v3(rqd[3], rqd[4], rqd[5]);
     const V3 Vw0 = mul(R0, w3), Vv0 = mul(R0, v3_);
-    const V3 tw = cross(an0, Vw0) + cross(af0, Vv0) + vw0, tv = cross(af0, Vw0) + vv0;
+    const V3 tw = cross(an, Vw0) + cross(af, Vv0) + vwb, tv = cross(af, Vw0) + vvb;
     const V3 bw = mulT(R0, tw), bv = mulT(R0, tv);
     const float add[6] = {bw.x, bw.y, bw.z, bv.x, bv.y, bv.z};
 #pragma unroll
     for (int j = 0; j < 6; ++j)
       if (lane == j) g.qdb += add[j];
-    const float4 a0 = lds4(w, ox), a1 = lds4(w, ox + 4);
-    const float2 a2 = *reinterpret_cast<const float2*>(&w[ox + 8]);
     M33 T;
-    T.m[0] = a0.x; T.m[1] = a0.y; T.m[2] = a0.z; T.m[3] = a0.w;
-    T.m[4] = a1.x; T.m[5] = a1.y; T.m[6] = a1.z; T.m[7] = a1.w; T.m[8] = a2.x;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) T.m[j] = xq[j];
     T = mul(T, R0);   // the root origin is the reference point (P = 0)
-    add_outer(T, Fn0, v3(-rl[0], -rl[1], -rl[2]));
-    add_outer(T, an0, v3(rqdd[0], rqdd[1], rqdd[2]));
+    add_outer(T, Fn, v3(-rl[0], -rl[1], -rl[2]));
+    add_outer(T, an, v3(rqdd[0], rqdd[1], rqdd[2]));
     add_outer(T, tw, w3);
-    add_outer(T, Ff0, v3(-rl[3], -rl[4], -rl[5]));
-    add_outer(T, af0, v3(rqdd[3], rqdd[4], rqdd[5]));
+    add_outer(T, Ff, v3(-rl[3], -rl[4], -rl[5]));
+    add_outer(T, af, v3(rqdd[3], rqdd[4], rqdd[5]));
     add_outer(T, tv, v3_);
     quat_to_R_adj(rx, ry, rz, rw, T, g.rqb[3], g.rqb[4], g.rqb[5], g.rqb[6]);
-    g.rqb[2] += w[ox + 12];
+    g.rqb[2] += xq[12];
   }
 }
 
