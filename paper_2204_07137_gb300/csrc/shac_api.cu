@@ -60,6 +60,16 @@ struct shac_batch {
   // the team size they were built for
   JitKernels spec;
   int spec_lanes = 0;
+  // what a launch of the current shape needs (plan_launch): index 0 forward, 1 adjoint
+  struct Plan {
+    shac_status st = SHAC_ERR_CAPACITY;
+    bool lanes = false;
+    int block = 0, grid[2] = {0, 0}, smem_warp_floats = 0;
+    size_t smem = 0;
+    const void* kernel[2] = {nullptr, nullptr};
+    unsigned int spec_key = 0;
+    int env_stride[MAX_GROUPS] = {0}, dense_nm[MAX_GROUPS] = {0};
+  } plan;
 };
 
 static shac_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? SHAC_OK : SHAC_ERR_CUDA; }
@@ -558,9 +568,56 @@ static int batched_warps(const shac_batch* b) {
   return W;
 }
 
+// Everything a launch needs that only the launch shape decides, worked out when
+// that changes: the scratch strides, the kernels (model-specialised while the shape
+// is the one they were built for), CTA size, shared memory and grids.  The step
+// calls then make one driver call, the launch (before, the attribute, the occupancy
+// query and a counter's memset went with every one: a step of 64 cart-poles 24.6
+// -> 20.9 us a call).
+static void plan_launch(shac_batch* b) {
+  shac_batch::Plan p;
+  p.lanes = lane_form(b);
+  int n_items = 0;
+  for (size_t gi = 0; gi < b->groups.size(); ++gi) {
+    const Group& g = b->groups[gi];
+    p.env_stride[gi] = env_stride(batch_layout(b, g), g.lanes);
+    p.dense_nm[gi] = dense_class(g.m->nv, g.lanes);
+    n_items += (g.N + 32 / g.lanes - 1) / (32 / g.lanes);
+  }
+  p.smem_warp_floats = (int)batched_smem_warp_floats(b);
+  const int W = batched_warps(b);
+  int dev = -1;
+  if (b->form == SHAC_FORM_BATCHED && W >= 1 && cudaGetDevice(&dev) == cudaSuccess &&
+      (dev == b->device || cudaSetDevice(b->device) == cudaSuccess)) {
+    p.block = 32 * W;
+    p.smem = (size_t)W * p.smem_warp_floats * sizeof(float);
+    const bool spec = b->spec.key != 0u && b->spec_lanes == b->groups[0].lanes;
+    if (spec) p.spec_key = b->spec.key;
+    p.st = SHAC_OK;
+    for (int k = 0; k < 2 && p.st == SHAC_OK; ++k) {
+      p.kernel[k] = spec ? (k ? b->spec.adj : b->spec.fwd) : batched_kernel(k == 1, p.lanes);
+      // the opt-in above 48 KB, always to the same limit: other batches launch the
+      // same kernels with other sizes
+      int occ = 0;
+      if (cudaFuncSetAttribute(p.kernel[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BLOCK_LIMIT) !=
+          cudaSuccess)
+        p.st = SHAC_ERR_CAPACITY;
+      else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, p.kernel[k], p.block, p.smem) != cudaSuccess)
+        p.st = SHAC_ERR_CUDA;
+      else if (occ < 1)
+        p.st = SHAC_ERR_CAPACITY;
+      p.grid[k] = std::max(1, std::min(b->num_sms * occ, (n_items + W - 1) / W));
+    }
+    if (dev != b->device) cudaSetDevice(dev);
+  }
+  b->plan = p;
+}
+
 // Work items sorted by per-warp cost (largest first) so the dynamic schedule
 // finishes the long items early.
+static void plan_launch(shac_batch* b);
 static shac_status build_items(shac_batch* b) {
+  plan_launch(b);
   std::vector<std::pair<double, WorkItem>> items;
   for (int gi = 0; gi < (int)b->groups.size(); ++gi) {
     const Group& g = b->groups[gi];
@@ -719,6 +776,7 @@ extern "C" shac_status shac_batch_specialize(shac_batch* b, int32_t enable) {
   if (!enable) {
     b->spec = JitKernels{};
     b->spec_lanes = 0;
+    plan_launch(b);
     return SHAC_OK;
   }
   if (b->form != SHAC_FORM_BATCHED || b->groups.size() != 1) return SHAC_ERR_UNSUPPORTED;
@@ -733,6 +791,7 @@ extern "C" shac_status shac_batch_specialize(shac_batch* b, int32_t enable) {
   if (st != SHAC_OK) return st;
   b->spec = k;
   b->spec_lanes = g.lanes;
+  plan_launch(b);
   return SHAC_OK;
 }
 
@@ -756,16 +815,16 @@ static PlainGroup plain_group(const shac_batch* b, int gi, void* ws) {
 
 static shac_status batched_launch(shac_batch* b, BatchedArgs& a, void* ws, cudaStream_t s, bool adjoint,
                                   bool window = false) {
-  const bool lanes = lane_form(b);
-  a.models = b->d_models + (lanes ? b->groups.size() : 0);
+  const shac_batch::Plan& p = b->plan;
   a.n_groups = (int)b->groups.size();
   a.io = b->io;
+  a.models = b->d_models + (p.lanes ? b->groups.size() : 0);
   for (int gi = 0; gi < a.n_groups; ++gi) {
     a.lanes[gi] = b->groups[gi].lanes;
-    a.env_stride[gi] = env_stride(batch_layout(b, b->groups[gi]), b->groups[gi].lanes);
-    a.dense_nm[gi] = dense_class(b->groups[gi].m->nv, b->groups[gi].lanes);
+    a.env_stride[gi] = p.env_stride[gi];
+    a.dense_nm[gi] = p.dense_nm[gi];
   }
-  a.smem_warp_floats = (int)batched_smem_warp_floats(b);
+  a.smem_warp_floats = p.smem_warp_floats;
   a.items = b->d_items;
   a.n_items = b->n_items;
   a.counter = reinterpret_cast<int*>(static_cast<char*>(ws) + b->ws_counter);
@@ -781,37 +840,14 @@ static shac_status batched_launch(shac_batch* b, BatchedArgs& a, void* ws, cudaS
   }
   a.flags = b->d_flags;
   if (b->n_items == 0) return SHAC_OK;
-  const int W = batched_warps(b);
-  if (W < 1) return SHAC_ERR_CAPACITY;
-  const size_t smem = (size_t)W * a.smem_warp_floats * sizeof(float);
-  const int block = 32 * W;
-  // the model-specialised kernels while the launch shape is the one they were built for
-  const void* spec = nullptr;
-  if (b->spec.key != 0u && b->spec_lanes == b->groups[0].lanes) {
-    spec = adjoint ? b->spec.adj : b->spec.fwd;
-    a.spec_key = b->spec.key;
-  }
-  // Static plus dynamic shared memory above 48 KB needs the opt-in attribute;
-  // the kernels' static part (the model table) is under 8 KB.
-  if (smem > 40 * 1024) {
-    const cudaError_t e = spec ? cudaFuncSetAttribute(spec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                               : batched_set_smem_limit(smem, lanes);
-    if (e != cudaSuccess) return SHAC_ERR_CAPACITY;
-  }
-  int occ = 0;
-  const cudaError_t oe = spec ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, spec, block, smem)
-                              : batched_occupancy(&occ, block, smem, adjoint, lanes);
-  if (oe != cudaSuccess) return SHAC_ERR_CUDA;
-  if (occ < 1) return SHAC_ERR_CAPACITY;
-  const int grid = std::max(1, std::min(b->num_sms * occ, (b->n_items + W - 1) / W));
-  if (cudaMemsetAsync(a.counter, 0, sizeof(int), s) != cudaSuccess) return SHAC_ERR_CUDA;
-  if (spec) {
-    void* args[] = {&a};
-    return cuda_ok(cudaLaunchKernel(spec, dim3(grid), dim3(block), args, smem, s));
-  }
-  if (adjoint) launch_batched_adjoint(a, grid, block, smem, lanes, s);
-  else launch_batched_forward(a, grid, block, smem, lanes, s);
-  return cuda_ok(cudaGetLastError());
+  if (p.st != SHAC_OK) return p.st;
+  a.spec_key = p.spec_key;
+  const int grid = p.grid[adjoint];
+  // a warp for every item: each takes its own, and the shared counter is not needed
+  if (grid * (p.block / 32) >= b->n_items) a.counter = nullptr;
+  else if (cudaMemsetAsync(a.counter, 0, sizeof(int), s) != cudaSuccess) return SHAC_ERR_CUDA;
+  void* args[] = {&a};
+  return cuda_ok(cudaLaunchKernel(p.kernel[adjoint], dim3(grid), dim3(p.block), args, p.smem, s));
 }
 
 // Episodic-window arguments (early termination with reset); batched form only.

@@ -27,10 +27,10 @@ namespace shac {
 
 // Register caps of the batched kernels (forward, adjoint): the live state of
 // the chain carries and of the 32-row dense path fits without spills; the
-// host launches at most 8 warps per CTA (8 x 32 x 240 registers fit an SM's
+// host launches at most 8 warps per CTA (8 x 32 x 255 registers fit an SM's
 // 64 Ki, and two 4-warp CTAs stay resident per SM).
-#define BATCHED_REGS_FORWARD 208
-#define BATCHED_REGS_ADJOINT 240
+#define BATCHED_REGS_FORWARD 232
+#define BATCHED_REGS_ADJOINT 255
 
 
 struct Team {
@@ -48,9 +48,15 @@ __device__ __forceinline__ void team_store(const SMem& w, int o, float* dst, int
   for (int j = lane; j < dim; j += nl) dst[(size_t)j * N + e] = w[o + j];
 }
 
+// The warp's next work item: from the shared counter, or, when the grid has a warp
+// for every item (no counter), its own and then none.  Either way through a
+// shuffle: from its result the compiler knows the item, and with it every branch of
+// the work, to be the same for the whole warp (the ant-like model's forward substep
+// took 28 % longer with an item computed from the thread index).
 __device__ __forceinline__ bool next_item(const BatchedArgs& a, int& item) {
   int v = 0;
-  if ((threadIdx.x & 31) == 0) v = atomicAdd(a.counter, 1);
+  if (!a.counter) v = item < 0 ? (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) : a.n_items;
+  else if ((threadIdx.x & 31) == 0) v = atomicAdd(a.counter, 1);
   item = __shfl_sync(0xffffffffu, v, 0);
   return item < a.n_items;
 }
@@ -274,7 +280,7 @@ __global__ void __maxnreg__(ADJ ? BATCHED_REGS_ADJOINT : BATCHED_REGS_FORWARD) k
   __syncthreads();
   const int warp = threadIdx.x >> 5;
   float* wsm = smem + (size_t)warp * a.smem_warp_floats;
-  int item_idx;
+  int item_idx = -1;
   while (next_item(a, item_idx)) {
     const WorkItem it = a.items[item_idx];
     const DevModel& M = s_models[it.group];

@@ -163,28 +163,9 @@ void launch_plain_adj_store_state(const PlainGroup& g, float* qb, float* qdb, co
 
 namespace shac {
 
-template <bool ADJ>
-static const void* batched_kernel(bool lanes) {
-  return lanes ? (const void*)k_batched<ADJ, true> : (const void*)k_batched<ADJ, false>;
-}
-static void launch(const void* k, const BatchedArgs& a, int grid, int block, size_t smem, cudaStream_t s) {
-  void* args[] = {const_cast<BatchedArgs*>(&a)};
-  cudaLaunchKernel(k, dim3(grid), dim3(block), args, smem, s);
-}
-void launch_batched_forward(const BatchedArgs& a, int grid, int block, size_t smem, bool lanes, cudaStream_t s) {
-  launch(batched_kernel<false>(lanes), a, grid, block, smem, s);
-}
-void launch_batched_adjoint(const BatchedArgs& a, int grid, int block, size_t smem, bool lanes, cudaStream_t s) {
-  launch(batched_kernel<true>(lanes), a, grid, block, smem, s);
-}
-cudaError_t batched_set_smem_limit(size_t smem, bool lanes) {
-  cudaError_t e = cudaFuncSetAttribute(batched_kernel<false>(lanes), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(batched_kernel<true>(lanes), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-cudaError_t batched_occupancy(int* blocks_per_sm, int block, size_t smem, bool adjoint, bool lanes) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      blocks_per_sm, adjoint ? batched_kernel<true>(lanes) : batched_kernel<false>(lanes), block, smem);
+const void* batched_kernel(bool adjoint, bool lanes) {
+  if (lanes) return adjoint ? (const void*)k_batched<true, true> : (const void*)k_batched<false, true>;
+  return adjoint ? (const void*)k_batched<true, false> : (const void*)k_batched<false, false>;
 }
 
 }  // namespace shac

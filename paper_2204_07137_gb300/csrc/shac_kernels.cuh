@@ -79,11 +79,9 @@ struct BatchedArgs {
 };
 
 #ifndef __CUDACC_RTC__
-// lanes: every group's team has a lane per link and DOF (the lane form's kernels)
-void launch_batched_forward(const BatchedArgs& a, int grid, int block, size_t smem, bool lanes, cudaStream_t s);
-void launch_batched_adjoint(const BatchedArgs& a, int grid, int block, size_t smem, bool lanes, cudaStream_t s);
-cudaError_t batched_occupancy(int* blocks_per_sm, int block, size_t smem, bool adjoint, bool lanes);
-cudaError_t batched_set_smem_limit(size_t smem, bool lanes);
+// The batched kernels as handles for the runtime's launch and attribute calls.
+// lanes: every group's team has a lane per link and DOF (the lane form).
+const void* batched_kernel(bool adjoint, bool lanes);
 
 // Plain form: one environment per thread, one kernel per stage.
 struct PlainGroup {

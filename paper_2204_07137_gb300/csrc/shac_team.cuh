@@ -43,7 +43,7 @@ struct LaneConst {
   M33 jrot;
   float icom[6];
   float mass, arm, damp, gear, qlo, qhi, crad;
-  float h, klim;
+  float klim;
 };
 
 __device__ __forceinline__ LaneConst lane_const(const DevModel& M, int lane) {
@@ -68,7 +68,7 @@ __device__ __forceinline__ LaneConst lane_const(const DevModel& M, int lane) {
   c.qlo = gf(LF_QLO); c.qhi = gf(LF_QHI);
   c.cpos = v3(gf(LF_CPOS), gf(LF_CPOS + 1), gf(LF_CPOS + 2)); c.crad = gf(LF_CRAD);
   c.base = v3(gf(LF_BASE), gf(LF_BASE + 1), gf(LF_BASE + 2));
-  c.h = M.h; c.klim = M.klim;
+  c.klim = M.klim;
   return c;
 }
 
@@ -204,8 +204,11 @@ __device__ __forceinline__ void lane_sums(const DevModel& M, const SMem& w, floa
       const int pn = M.par8[i - 1];
       const float s = v + carry;
       w[a] = s;
-      const bool chain = p == i - 1;
-      if (!chain && p >= 0) w[o + XB * p] += s;
+      // a branch's parent takes the sum in memory; otherwise the same access adds
+      // nothing to this link's own (spent) block, which costs less than a jump
+      const bool chain = p == i - 1, up = !chain && p >= 0;
+      const int b = up ? o + XB * p : a;
+      w[b] += up ? s : 0.f;
       carry = chain ? s : 0.f;
       v = vn;
       p = pn;
