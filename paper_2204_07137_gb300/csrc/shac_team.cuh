@@ -19,9 +19,9 @@
 // substep costs its dependent instructions, not its arithmetic.  The per-link
 // passes over shared-memory scratch that this form replaces cost a store, a
 // barrier and a load between any two of them.  Measured on the ant-like model,
-// specialised, a substep's cycles (T = 16): forward 10.8 k -> 4.9 k, reverse
-// 11.5 k -> 5.3 k; forward + adjoint of 2048 environments, h = 8: 2.09 -> 1.09 ms;
-// the generic kernels on 1531 environments, h = 2: 0.98 -> 0.47 ms.
+// specialised, a substep's cycles (T = 16): forward 10.8 k -> 4.4 k, reverse
+// 11.5 k -> 5.0 k; forward + adjoint of 2048 environments, h = 8: 2.09 -> 0.98 ms;
+// the generic kernels on 1531 environments, h = 2: 0.98 -> 0.43 ms.
 #pragma once
 #include "shac_device.cuh"
 
@@ -517,8 +517,8 @@ constexpr int SEG_GROUP = 2;
 // mrows conflict-free steps whatever the distribution of the items over the
 // links (a lane per link takes as many steps as the busiest link has items: 99
 // of the 152-muscle model's 608, where 22 rows serve).  The unused places hold
-// zeros.  512 environments of that model, h = 2: 7.27 -> 1.81 ms, the scratch of
-// an environment down from 50 to 35 KB, so that all of them are resident.  Planes of MSLOTS * mrows floats: points x y z at o_MX, forces (reverse:
+// zeros.  512 environments of that model, h = 2: 7.27 -> 1.41 ms, the scratch of
+// an environment down from 60 to 36 KB, so that all of them are resident.  Planes of MSLOTS * mrows floats: points x y z at o_MX, forces (reverse:
 // the points' cotangents) x y z at o_MF.
 __device__ __forceinline__ void muscle_clear(const DevModel& M, const SMem& w, int lane, int nl) {
   zero_range(w, M.o_MX, 3 * MSLOTS * M.mrows, lane, nl);
