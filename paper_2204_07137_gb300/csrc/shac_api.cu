@@ -23,7 +23,7 @@ struct shac_model {
       dof_k,
       dof_act, item_link, seg_mus, mus_seg_ptr, anc_mask, chain_tail, ln_i, ms_ptr, sg_place;
   std::vector<float> axis, jpos, jrot, mass, com, icom, qlo, qhi, arm, damp, gear, item_pos, crad, fmax, rwq, rwqd, ln_f, sg_f;
-  int lanes_needed = 0, nround = 0, mrows = 0;
+  int lanes_needed = 0, nround = 0, deepest = 0, mrows = 0;
   DevModel layout, lane_layout;   // sizes + scratch offsets (pointers unset): general and lane form
 };
 
@@ -151,6 +151,7 @@ static void compute_lanes(shac_model* m) {
   compute_muscle_slots(m);
   m->nround = 0;
   while ((1 << m->nround) < deepest + 1) ++m->nround;
+  m->deepest = deepest;
   m->ln_i.assign(LI_N * LANE_COLS, 0);
   m->ln_f.assign(LF_N * LANE_COLS, 0.f);
   if (next > LANE_COLS) return;
@@ -165,6 +166,7 @@ static void compute_lanes(shac_model* m) {
     const int l = lane_of[i];
     I(LI_LINK, l) = i; I(LI_JT, l) = m->jtype[i]; I(LI_Q, l) = m->qs[i];
     I(LI_C0, l) = m->lc_ptr[i]; I(LI_C1, l) = m->lc_ptr[i + 1];
+    I(LI_DEPTH, l) = level[i];
     unsigned anc = 0;                     // the 2^r-th ancestors' lanes, 6 bits each (63: none)
     for (int r = 0; r < 5; ++r) {
       int j = i;
@@ -191,6 +193,7 @@ static void compute_lanes(shac_model* m) {
   for (int d = 0; d < nv; ++d) {
     I(LI_DLINK, d) = m->dof_link[d];
     I(LI_ACT, d) = m->dof_act[d];
+    I(LI_ROW, d) = m->anc_mask[d];
     for (int a = 0; a < nv; ++a)          // DOF a moves with d: an entry of d's row of the upper triangle
       if (((unsigned)m->anc_mask[a] >> d) & 1u) I(LI_DESC, d) |= (int)(1u << a);
     F(LF_ARM, d) = m->arm[d]; F(LF_DAMP, d) = m->damp[d]; F(LF_GEAR, d) = m->gear[d];
@@ -223,6 +226,7 @@ static void compute_layout(shac_model* m) {
   take(d.o_QC, m->nq); take(d.o_QDC, nv); take(d.o_LW, LWORK * L);
   d.lanes_needed = m->lanes_needed;
   d.nround = m->nround;
+  d.deepest = m->deepest;
   d.mrows = m->mrows;
   for (int i = 0; i < std::min(L, 32); ++i) d.par8[i] = (signed char)m->parent[i];
   take(d.o_B, nv); take(d.o_T, nv);

@@ -95,8 +95,9 @@ struct DevModel {
   // reward weights
   const float *rwq, *rwqd;
   // lane form (shac_team.cuh): lanes a team needs (DOFs, then the links without
-  // one), doubling rounds, and the lane columns of the model's constants
-  int lanes_needed, nround;
+  // one), doubling rounds, the deepest link's level, and the lane columns of the
+  // model's constants
+  int lanes_needed, nround, deepest;
   signed char par8[32];                  // link parents (models of at most 32 links)
   const int* ln_i;
   const float* ln_f;
@@ -204,15 +205,24 @@ __device__ __forceinline__ void team_sync(int nl) {
 }
 
 // ----------------------------------------------------------- small math --
+// Sums of two and three products with their roundings fixed here.  Left to the
+// compiler, which of the products joins a fused multiply-add depends on the code
+// around the inlined expression; then two kernels with the same source lines round
+// differently, and a contact or friction test can fall differently in them.
+__device__ __forceinline__ float sum2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ float diff2(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
+__device__ __forceinline__ float sum3(float a, float b, float c, float d, float e, float f) {
+  return __fmaf_rn(e, f, sum2(a, b, c, d));
+}
 struct V3 { float x, y, z; };
 __device__ __forceinline__ V3 v3(float a, float b, float c) { return {a, b, c}; }
 __device__ __forceinline__ V3 operator+(V3 a, V3 b) { return {a.x + b.x, a.y + b.y, a.z + b.z}; }
 __device__ __forceinline__ V3 operator-(V3 a, V3 b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
 __device__ __forceinline__ V3 operator-(V3 a) { return {-a.x, -a.y, -a.z}; }
 __device__ __forceinline__ V3 operator*(float s, V3 a) { return {s * a.x, s * a.y, s * a.z}; }
-__device__ __forceinline__ float dot(V3 a, V3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+__device__ __forceinline__ float dot(V3 a, V3 b) { return sum3(a.x, b.x, a.y, b.y, a.z, b.z); }
 __device__ __forceinline__ V3 cross(V3 a, V3 b) {
-  return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+  return {diff2(a.y, b.z, a.z, b.y), diff2(a.z, b.x, a.x, b.z), diff2(a.x, b.y, a.y, b.x)};
 }
 template <class Mem> __device__ __forceinline__ V3 ld3(const Mem& w, int o) { return {w[o], w[o + 1], w[o + 2]}; }
 template <class Mem> __device__ __forceinline__ void st3(const Mem& w, int o, V3 v) { w[o] = v.x; w[o + 1] = v.y; w[o + 2] = v.z; }
@@ -237,12 +247,12 @@ __device__ __forceinline__ M33 cldm(const float* p) {
   return r;
 }
 __device__ __forceinline__ V3 mul(const M33& R, V3 x) {
-  return {R.m[0] * x.x + R.m[1] * x.y + R.m[2] * x.z, R.m[3] * x.x + R.m[4] * x.y + R.m[5] * x.z,
-          R.m[6] * x.x + R.m[7] * x.y + R.m[8] * x.z};
+  return {sum3(R.m[0], x.x, R.m[1], x.y, R.m[2], x.z), sum3(R.m[3], x.x, R.m[4], x.y, R.m[5], x.z),
+          sum3(R.m[6], x.x, R.m[7], x.y, R.m[8], x.z)};
 }
 __device__ __forceinline__ V3 mulT(const M33& R, V3 x) {
-  return {R.m[0] * x.x + R.m[3] * x.y + R.m[6] * x.z, R.m[1] * x.x + R.m[4] * x.y + R.m[7] * x.z,
-          R.m[2] * x.x + R.m[5] * x.y + R.m[8] * x.z};
+  return {sum3(R.m[0], x.x, R.m[3], x.y, R.m[6], x.z), sum3(R.m[1], x.x, R.m[4], x.y, R.m[7], x.z),
+          sum3(R.m[2], x.x, R.m[5], x.y, R.m[8], x.z)};
 }
 __device__ __forceinline__ M33 mul(const M33& A, const M33& B) {
   M33 C;
@@ -250,7 +260,7 @@ __device__ __forceinline__ M33 mul(const M33& A, const M33& B) {
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-      C.m[3 * i + j] = A.m[3 * i] * B.m[j] + A.m[3 * i + 1] * B.m[3 + j] + A.m[3 * i + 2] * B.m[6 + j];
+      C.m[3 * i + j] = sum3(A.m[3 * i], B.m[j], A.m[3 * i + 1], B.m[3 + j], A.m[3 * i + 2], B.m[6 + j]);
   return C;
 }
 __device__ __forceinline__ M33 mulBT(const M33& A, const M33& B) {   // A B^T
@@ -259,7 +269,7 @@ __device__ __forceinline__ M33 mulBT(const M33& A, const M33& B) {   // A B^T
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-      C.m[3 * i + j] = A.m[3 * i] * B.m[3 * j] + A.m[3 * i + 1] * B.m[3 * j + 1] + A.m[3 * i + 2] * B.m[3 * j + 2];
+      C.m[3 * i + j] = sum3(A.m[3 * i], B.m[3 * j], A.m[3 * i + 1], B.m[3 * j + 1], A.m[3 * i + 2], B.m[3 * j + 2]);
   return C;
 }
 __device__ __forceinline__ V3 col(const M33& R, int k) { return {R.m[k], R.m[3 + k], R.m[6 + k]}; }
@@ -267,9 +277,9 @@ __device__ __forceinline__ V3 col(const M33& R, int k) { return {R.m[k], R.m[3 +
 // unit-quaternion (x, y, z, w) rotation matrix
 __device__ __forceinline__ M33 quat_to_R(float x, float y, float z, float w) {
   M33 R;
-  R.m[0] = 1.f - 2.f * (y * y + z * z); R.m[1] = 2.f * (x * y - z * w); R.m[2] = 2.f * (x * z + y * w);
-  R.m[3] = 2.f * (x * y + z * w); R.m[4] = 1.f - 2.f * (x * x + z * z); R.m[5] = 2.f * (y * z - x * w);
-  R.m[6] = 2.f * (x * z - y * w); R.m[7] = 2.f * (y * z + x * w); R.m[8] = 1.f - 2.f * (x * x + y * y);
+  R.m[0] = 1.f - 2.f * (__fmul_rn(y, y) + __fmul_rn(z, z)); R.m[1] = 2.f * diff2(x, y, z, w); R.m[2] = 2.f * sum2(x, z, y, w);
+  R.m[3] = 2.f * sum2(x, y, z, w); R.m[4] = 1.f - 2.f * sum2(x, x, z, z); R.m[5] = 2.f * diff2(y, z, x, w);
+  R.m[6] = 2.f * diff2(x, z, y, w); R.m[7] = 2.f * sum2(y, z, x, w); R.m[8] = 1.f - 2.f * sum2(x, x, y, y);
   return R;
 }
 // adjoint of quat_to_R: accumulate dR : Rbar into (xb, yb, zb, wb)
@@ -287,21 +297,33 @@ __device__ __forceinline__ M33 axis_angle(V3 a, float t) {
   sincosf(t, &s, &c);
   float k = 1.f - c;
   M33 R;
-  R.m[0] = c + k * a.x * a.x; R.m[1] = k * a.x * a.y - s * a.z; R.m[2] = k * a.x * a.z + s * a.y;
-  R.m[3] = k * a.y * a.x + s * a.z; R.m[4] = c + k * a.y * a.y; R.m[5] = k * a.y * a.z - s * a.x;
-  R.m[6] = k * a.z * a.x - s * a.y; R.m[7] = k * a.z * a.y + s * a.x; R.m[8] = c + k * a.z * a.z;
+  R.m[0] = c + k * a.x * a.x; R.m[1] = diff2(k * a.x, a.y, s, a.z); R.m[2] = sum2(k * a.x, a.z, s, a.y);
+  R.m[3] = sum2(k * a.y, a.x, s, a.z); R.m[4] = c + k * a.y * a.y; R.m[5] = diff2(k * a.y, a.z, s, a.x);
+  R.m[6] = diff2(k * a.z, a.x, s, a.y); R.m[7] = sum2(k * a.z, a.y, s, a.x); R.m[8] = c + k * a.z * a.z;
   return R;
 }
 
 // spatial inertia at the world origin, 10 floats: m, h = m c (3), Io (xx yy zz xy xz yz)
+// of a body of mass m at c with the rotated inertia Iw (roundings fixed as above)
+__device__ __forceinline__ void spatial_inertia(const M33& Iw, float m, V3 c, float (&si)[10]) {
+  const float cc = dot(c, c);
+  const V3 h = m * c;
+  si[0] = m; si[1] = h.x; si[2] = h.y; si[3] = h.z;
+  si[4] = __fmaf_rn(m, __fmaf_rn(-c.x, c.x, cc), Iw.m[0]);
+  si[5] = __fmaf_rn(m, cc - __fmul_rn(c.y, c.y), Iw.m[4]);
+  si[6] = __fmaf_rn(m, __fmaf_rn(-c.z, c.z, cc), Iw.m[8]);
+  si[7] = __fmaf_rn(-h.x, c.y, Iw.m[1]);
+  si[8] = __fmaf_rn(-h.x, c.z, Iw.m[2]);
+  si[9] = __fmaf_rn(-h.y, c.z, Iw.m[5]);
+}
 // product I * (w, v) = (Io w + h x v, m v - h x w)
 template <class Mem>
 __device__ __forceinline__ void si_mul(const Mem& w, int o, V3 xw, V3 xv, V3& yn, V3& yf) {
   float m = w[o];
   V3 h = ld3(w, o + 1);
   float ixx = w[o + 4], iyy = w[o + 5], izz = w[o + 6], ixy = w[o + 7], ixz = w[o + 8], iyz = w[o + 9];
-  V3 Iw = {ixx * xw.x + ixy * xw.y + ixz * xw.z, ixy * xw.x + iyy * xw.y + iyz * xw.z,
-           ixz * xw.x + iyz * xw.y + izz * xw.z};
+  V3 Iw = {sum3(ixx, xw.x, ixy, xw.y, ixz, xw.z), sum3(iyy, xw.y, ixy, xw.x, iyz, xw.z),
+           sum3(ixz, xw.x, iyz, xw.y, izz, xw.z)};
   yn = Iw + cross(h, xv);
   yf = m * xv - cross(h, xw);
 }
@@ -432,7 +454,7 @@ __device__ __forceinline__ void poses_by_rows(const DevModel& M, const Mem& w, i
       if (p >= 0) {
         const int op = lrec(M, p);
         const V3 rp = ld3(w, op + LR_R + 3 * r);
-        row = rp.x * ld3(w, ol + LR_R) + rp.y * ld3(w, ol + LR_R + 3) + rp.z * ld3(w, ol + LR_R + 6);
+        row = mulT(ldm(w, ol + LR_R), rp);
         pr = w[op + LR_P + r] + dot(rp, ld3(w, ol + LR_P));
       }
       st3(w, o + LR_R + 3 * r, row);
@@ -578,11 +600,10 @@ __device__ __forceinline__ void lk_local(const DevModel& M, const Mem& w, int i)
   const float m = __ldg(M.mass + i);
   const V3 c = P + mul(R, cld3(M.com + 3 * i));
   const M33 Iw = mulBT(mul(R, com_inertia(M, i)), R);
-  const float cc = dot(c, c);
-  const V3 h = m * c;
-  const float ixx = Iw.m[0] + m * (cc - c.x * c.x), iyy = Iw.m[4] + m * (cc - c.y * c.y);
-  const float izz = Iw.m[8] + m * (cc - c.z * c.z), ixy = Iw.m[1] - m * c.x * c.y;
-  const float ixz = Iw.m[2] - m * c.x * c.z, iyz = Iw.m[5] - m * c.y * c.z;
+  float si[10];
+  spatial_inertia(Iw, m, c, si);
+  const V3 h = v3(si[1], si[2], si[3]);
+  const float ixx = si[4], iyy = si[5], izz = si[6], ixy = si[7], ixz = si[8], iyz = si[9];
   {   // the link's own spatial inertia, in the record and as the start of its composite inertia
     const int o = lrec(M, i) + LR_SI, oc = lwork(M, i) + LW_IC;
     w[o] = m; st3(w, o + 1, h);
@@ -591,8 +612,8 @@ __device__ __forceinline__ void lk_local(const DevModel& M, const Mem& w, int i)
     w[oc + 4] = ixx; w[oc + 5] = iyy; w[oc + 6] = izz; w[oc + 7] = ixy; w[oc + 8] = ixz; w[oc + 9] = iyz;
   }
   auto imul = [&](V3 xw, V3 xv, V3& yn, V3& yf) {
-    yn = v3(ixx * xw.x + ixy * xw.y + ixz * xw.z, ixy * xw.x + iyy * xw.y + iyz * xw.z,
-            ixz * xw.x + iyz * xw.y + izz * xw.z) + cross(h, xv);
+    yn = v3(sum3(ixx, xw.x, ixy, xw.y, ixz, xw.z), sum3(ixy, xw.x, iyy, xw.y, iyz, xw.z),
+            sum3(ixz, xw.x, iyz, xw.y, izz, xw.z)) + cross(h, xv);
     yf = m * xv - cross(h, xw);
   };
   // Sec. 3.1 contact model on the ground plane z = 0 (n = +z) for the contact
@@ -612,7 +633,7 @@ __device__ __forceinline__ void lk_local(const DevModel& M, const Mem& w, int i)
       if (d < 0.f) {
         const V3 vp = Vv + cross(Vw, x);
         const float fn = (-M.ke + M.kd * vp.z) * d;
-        const float vt = sqrtf(vp.x * vp.x + vp.y * vp.y);
+        const float vt = sqrtf(sum2(vp.x, vp.x, vp.y, vp.y));
         const float afn = fabsf(fn);
         if (M.kt * vt <= M.mu * afn) { f.x = -M.kt * vp.x; f.y = -M.kt * vp.y; }
         else { const float sc = M.mu * afn / vt; f.x = -sc * vp.x; f.y = -sc * vp.y; }
@@ -1345,8 +1366,8 @@ __device__ __forceinline__ void lk_adj_local(const DevModel& M, const Mem& w, in
   const float ixx = w[osi + 4], iyy = w[osi + 5], izz = w[osi + 6], ixy = w[osi + 7], ixz = w[osi + 8],
               iyz = w[osi + 9];
   auto imul = [&](V3 xw, V3 xv, V3& yn, V3& yf) {
-    yn = v3(ixx * xw.x + ixy * xw.y + ixz * xw.z, ixy * xw.x + iyy * xw.y + iyz * xw.z,
-            ixz * xw.x + iyz * xw.y + izz * xw.z) + cross(h, xv);
+    yn = v3(sum3(ixx, xw.x, ixy, xw.y, ixz, xw.z), sum3(ixy, xw.x, iyy, xw.y, iyz, xw.z),
+            sum3(ixz, xw.x, iyz, xw.y, izz, xw.z)) + cross(h, xv);
     yf = m * xv - cross(h, xw);
   };
   const V3 Vw = ld3(w, lrec(M, i) + LR_V), Vv = ld3(w, lrec(M, i) + LR_V + 3);
@@ -1416,7 +1437,7 @@ __device__ __forceinline__ void lk_adj_local(const DevModel& M, const Mem& w, in
       V3 xb = cross(f, neb);
       const V3 vp = Vv + cross(Vw, x);
       const float fn = f.z;
-      const float vt = sqrtf(vp.x * vp.x + vp.y * vp.y);
+      const float vt = sqrtf(sum2(vp.x, vp.x, vp.y, vp.y));
       const float afn = fabsf(fn);
       float fnb = fbar.z;
       V3 vpb = v3(0.f, 0.f, 0.f);

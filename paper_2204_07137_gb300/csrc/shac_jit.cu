@@ -53,7 +53,7 @@ const Field kFields[] = {
     {"o_RDB", &DevModel::o_RDB}, {"o_X", &DevModel::o_X}, {"o_R", &DevModel::o_R},
     {"o_MP", &DevModel::o_MP}, {"o_MB", &DevModel::o_MB}, {"o_MX", &DevModel::o_MX}, {"o_MF", &DevModel::o_MF},
     {"mrows", &DevModel::mrows}, {"lanes_needed", &DevModel::lanes_needed},
-    {"nround", &DevModel::nround}, {"rec_floats", &DevModel::rec_floats}, {"env_floats", &DevModel::env_floats},
+    {"nround", &DevModel::nround}, {"deepest", &DevModel::deepest}, {"rec_floats", &DevModel::rec_floats}, {"env_floats", &DevModel::env_floats},
 };
 
 // Replace every `M.<field>` (as a whole word) by the field's value.

@@ -8,36 +8,54 @@
 // right-hand vectors of the mass matrix, and the factor's transpose.
 //
 //   poses, velocities, accelerations: sums and products along each link's path
-//     to the root, by pointer doubling: in round r a lane combines its value with
-//     that of its 2^r-th ancestor (shuffles; ceil(log2(levels)) rounds);
+//     to the root by shuffles: a specialised build (and the reverse pass) by pointer
+//     doubling, in round r a lane combining its value with that of its 2^r-th ancestor
+//     (ceil(log2(levels)) rounds); the generic build a level of the tree a round;
 //   composite inertias and total forces: subtree sums, one component per lane;
-//   M = L^T L, eliminated leaves first (the last DOF first), so L has no entry
-//     outside the pairs (DOF, ancestor DOF): a specialised build, which knows the
-//     ancestors, skips the others and factors the DOFs of one tree level together.
+//   specialised: M = L^T L, eliminated leaves first (the last DOF first), so L has no
+//     entry outside the pairs (DOF, ancestor DOF): a specialised build, which knows
+//     the ancestors, skips the others and factors the DOFs of one tree level together;
+//   generic: M = L L^T, root first.
+//
+// The generic build's forward substep does the general kernels' operations in their
+// order (but for the muscles' sums), so a model has the same states, bit for bit, in
+// both forms.  A window's gradients jump where a contact, friction or limit switch is
+// decided by rounding; with other roundings one of some 80,000 environments came out
+// with a gradient some percent off the general kernels' (2 % of the batches of 1531
+// ant-like environments over two steps), with the same roundings none.  It costs the
+// generic windows about a tenth (1531 environments, h = 8: 1.67 -> 1.84 ms; the general
+// kernels 3.97; the deeper humanoid-like model 7.3 -> 8.8; 19.8).
 //
 // What bounds it is latency: at 2048 environments an SM holds seven warps, so a
 // substep costs its dependent instructions, not its arithmetic.  The per-link
 // passes over shared-memory scratch that this form replaces cost a store, a
 // barrier and a load between any two of them.  Measured on the ant-like model,
-// specialised, a substep's cycles (T = 16): forward 10.8 k -> 4.4 k, reverse
-// 11.5 k -> 5.0 k; forward + adjoint of 2048 environments, h = 8: 2.09 -> 0.98 ms;
-// the generic kernels on 1531 environments, h = 2: 0.98 -> 0.43 ms.
+// specialised, a substep's cycles (T = 16): forward 10.8 k -> 4.6 k, reverse
+// 11.5 k -> 5.0 k; forward + adjoint of 2048 environments, h = 8: 2.09 -> 1.00 ms;
+// the generic kernels on 1531 environments, h = 2: 0.98 -> 0.48 ms.
 #pragma once
 #include "shac_device.cuh"
 
 namespace shac {
 
 // This lane's share of the model (DevModel::ln_i, ln_f: one column per lane).
-enum { LI_LINK = 0, LI_JT, LI_ANC, LI_Q, LI_ACT, LI_C0, LI_C1, LI_DESC, LI_DLINK, LI_N };
+enum { LI_LINK = 0, LI_JT, LI_ANC, LI_Q, LI_ACT, LI_C0, LI_C1, LI_DESC, LI_ROW, LI_DLINK, LI_DEPTH, LI_N };
 enum { LF_AXIS = 0, LF_JROT = 3, LF_JPOS = 12, LF_COM = 15, LF_ICOM = 18, LF_MASS = 24, LF_ARM, LF_DAMP, LF_GEAR,
        LF_QLO, LF_QHI, LF_CPOS, LF_CRAD = LF_CPOS + 3, LF_BASE, LF_N = LF_BASE + 3 };
 constexpr int LANE_COLS = 32;
+// A row of the mass matrix on its lane: up the tree in the generic build, down it
+// in a specialised one (see Dense).
+#ifdef SHAC_SPEC_ANC
+constexpr int MASS_COLS = LI_DESC;
+#else
+constexpr int MASS_COLS = LI_ROW;
+#endif
 constexpr float MIN_NORMAL = 1.17549435e-38f;
 constexpr int MSLOTS = 32;   // columns of the muscles' via-point items
 
 struct LaneConst {
-  int link, jt, qi, act, c0, c1, dlink, ms0, ms1;
-  unsigned anc, desc;
+  int link, jt, qi, act, c0, c1, dlink, depth, ms0, ms1;
+  unsigned anc, cols;   // cols: entries of the lane's mass-matrix row
   bool own;             // lane < nv
   V3 axis, jpos, com, cpos, base;   // cpos, crad: the link's first contact; base: -g on a root link
   M33 jrot;
@@ -53,7 +71,8 @@ __device__ __forceinline__ LaneConst lane_const(const DevModel& M, int lane) {
   auto gf = [&](int k) { return __ldg(F + LANE_COLS * k); };
   LaneConst c;
   c.link = gi(LI_LINK); c.jt = gi(LI_JT); c.anc = (unsigned)gi(LI_ANC); c.qi = gi(LI_Q); c.act = gi(LI_ACT);
-  c.c0 = gi(LI_C0); c.c1 = gi(LI_C1); c.desc = (unsigned)gi(LI_DESC); c.dlink = gi(LI_DLINK);
+  c.c0 = gi(LI_C0); c.c1 = gi(LI_C1); c.cols = (unsigned)gi(MASS_COLS); c.dlink = gi(LI_DLINK);
+  c.depth = gi(LI_DEPTH);
   c.ms0 = c.ms1 = 0;
   if (M.nseg > 0 && c.link >= 0) { c.ms0 = __ldg(M.ms_ptr + c.link); c.ms1 = __ldg(M.ms_ptr + c.link + 1); }
   c.own = lane < M.nv;
@@ -86,14 +105,25 @@ __device__ __forceinline__ V3 team_shfl(V3 x, int src, int nl) {
   return v3(team_shfl(x.x, src, nl), team_shfl(x.y, src, nl), team_shfl(x.z, src, nl));
 }
 
-// Sums of x along the path to the root (own value included), by doubling.
-__device__ __forceinline__ void path_sums(const DevModel& M, unsigned anc, int nl, V3& a, V3& b) {
+// Sums of a and b along the path to the root (own value included) in the forward
+// substep.  A specialised build doubles.  The generic build takes the levels of the
+// tree in turn, the links of level r adding their parents': the general kernels' order
+// of additions, so that states come out the same to the last bit in both.
+__device__ __forceinline__ void path_sums(const DevModel& M, const LaneConst& c, int nl, V3& a, V3& b) {
+#ifdef SHAC_SPEC_ANC
 #pragma unroll
   for (int r = 0; r < M.nround; ++r) {
-    const unsigned s = (anc >> (6 * r)) & 63u;
+    const unsigned s = (c.anc >> (6 * r)) & 63u;
     const V3 pa = team_shfl(a, (int)(s & 31u), nl), pb = team_shfl(b, (int)(s & 31u), nl);
     if (s < 32u) { a = a + pa; b = b + pb; }
   }
+#else
+  const int src = (int)(c.anc & 31u);
+  for (int r = 1; r <= M.deepest; ++r) {
+    const V3 pa = team_shfl(a, src, nl), pb = team_shfl(b, src, nl);
+    if (c.depth == r) { a = a + pa; b = b + pb; }
+  }
+#endif
 }
 
 // 1 / sqrt(x) to 2 ulp, a subnormal x taken as zero: rsqrtf without the scaling
@@ -229,10 +259,75 @@ __device__ __forceinline__ void lane_sums(const DevModel& M, const SMem& w, floa
   team_sync(nl);   // the blocks are free again
 }
 
-// Which entries of the factor exist, and which DOFs may be eliminated
-// together: a specialised build has the ancestor masks as literals, the generic
-// build takes every pair and one DOF at a time.
+// Assembly of the lane's row of M + diag(arm) and the factor's rows in the record,
+// common to both eliminations below.
+template <int NM>
+struct DenseRows {
+  static constexpr int ST = dense_stride(NM);
+  // row[b] = (xw, xv) . (vector of DOF b at of) for the columns in c.cols, zero
+  // elsewhere; lanes from nv on: identity rows.
+  // The columns go in groups whose vectors are all read before the first product
+  // (one at a time, every column waited for its own reads: 54 cycles each).
+  static constexpr int GROUP = 7;
+  template <int B0, int... B>
+  static __device__ __forceinline__ void assemble_group(const SMem& w, int of, V3 sw, V3 sv, const LaneConst& c,
+                                                        int lane, float (&row)[NM], float& diag, iseq<B...>) {
+    float4 f0[sizeof...(B)];
+    float2 f1[sizeof...(B)];
+    ([&] {
+      f0[B] = lds4(w, of + XF * (B0 + B));
+      f1[B] = *reinterpret_cast<const float2*>(&w[of + XF * (B0 + B) + 4]);
+    }(), ...);
+    ([&] {
+      const float p = dot(sw, v3(f0[B].x, f0[B].y, f0[B].z)) + dot(sv, v3(f0[B].w, f1[B].x, f1[B].y));
+      float v = ((c.cols >> (B0 + B)) & 1u) ? p : 0.f;
+      if (B0 + B == lane) { v += c.arm; diag = v; }
+      row[B0 + B] = v;
+    }(), ...);
+  }
+  template <int B0 = 0>
+  static __device__ __forceinline__ void assemble(const SMem& w, int of, V3 sw, V3 sv, const LaneConst& c, int lane,
+                                                  float (&row)[NM], float& diag) {
+    if constexpr (B0 < NM) {
+      assemble_group<B0>(w, of, sw, sv, c, lane, row, diag, make_iseq<(NM - B0 < GROUP ? NM - B0 : GROUP)>{});
+      assemble<B0 + GROUP>(w, of, sw, sv, c, lane, row, diag);
+    }
+  }
+  // One lane's row of the factor (in the form ls) to the record: 16 bytes of every
+  // row side by side.
+  static __device__ __forceinline__ void store_row(float* fac, int rs, const float (&ls)[NM], int lane) {
+#pragma unroll
+    for (int k = 0; k < (NM + 3) / 4; ++k)
+      stg4(fac + 4 * (k * rs + lane), ls[4 * k], 4 * k + 1 < NM ? ls[4 * k + 1 < NM ? 4 * k + 1 : 0] : 0.f,
+           4 * k + 2 < NM ? ls[4 * k + 2 < NM ? 4 * k + 2 : 0] : 0.f,
+           4 * k + 3 < NM ? ls[4 * k + 3 < NM ? 4 * k + 3 : 0] : 0.f);
+  }
+  // The record's factor: entries k > lane of this lane's column and, below, all of
+  // its row (both zero elsewhere).
+  static __device__ __forceinline__ void load_record(const SMem& w, int of, int rs, int n, int lane, float (&lc)[NM],
+                                                     float (&ls)[NM]) {
+    const int oc = of + 4 * (lane >> 2) * rs + (lane & 3);
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {
+      const bool use = lane < k && k < n;
+      const float v = w[use ? oc + 4 * k : of];
+      lc[k] = use ? v : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < (NM + 3) / 4; ++k) {
+      const float4 v = lds4(w, of + 4 * (k * rs + (lane < n ? lane : 0)));
+      const float t[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (4 * k + j < NM) ls[4 * k + j < NM ? 4 * k + j : 0] = lane < n ? t[j] : 0.f;
+    }
+  }
+};
+
 #ifdef SHAC_SPEC_ANC
+// A specialised build eliminates leaves first, M = L^T L.  It has the ancestor masks
+// as literals, so it knows which entries of the factor exist and which DOFs may be
+// eliminated together.
 constexpr unsigned kAncMask[] = {SHAC_SPEC_ANC};
 constexpr int kAncCount = sizeof(kAncMask) / sizeof(kAncMask[0]);
 __host__ __device__ constexpr bool has_entry(int k, int j) { return k < kAncCount && j < k && ((kAncMask[k] >> j) & 1u); }
@@ -242,20 +337,18 @@ __host__ __device__ constexpr int dof_level(int k) {   // number of ancestors
   for (int b = 0; b < 32; ++b) n += (kAncMask[k] >> b) & 1u;
   return n;
 }
-#else
-__host__ __device__ constexpr bool has_entry(int k, int j) { return j < k; }
-__host__ __device__ constexpr int dof_level(int k) { return k; }
-#endif
 
 // Lane a holds row[b] = M_ab for its descendants b >= a (and itself), its
 // diagonal in diag and the right-hand side in b.  Eliminating DOF k: L_kk =
 // sqrt(pivot), L_ka = M_ak / L_kk on lane a, M_aj -= L_ka L_kj, and the forward
 // substitution y_k = b_k / L_kk, b_a -= L_ka y_k in the same pass.  L_ka goes to
 // row k of the factor in shared memory, where lane k reads it for the backward
-// substitution and the record keeps it for the adjoint.
+// substitution and the record keeps it for the adjoint: the unit factor, row k
+// holding L_kj / L_kk for j < k, next to 1 / L_kk.
 template <int NM>
-struct Dense {
-  static constexpr int ST = dense_stride(NM);
+struct Dense : DenseRows<NM> {
+  using Rows = DenseRows<NM>;
+  static constexpr int ST = Rows::ST;
   template <int K, int J>
   static __device__ __forceinline__ void update(float (&row)[NM], float lk, int nl) {
     if constexpr (has_entry(K, J)) row[J] = fmaf(-lk, team_shfl(lk, J, nl), row[J]);
@@ -267,7 +360,7 @@ struct Dense {
   template <int LV, int K>
   static __device__ __forceinline__ void pivot(float diag, float (&inv)[NM], float b, float (&y)[NM], int nl) {
     if constexpr (dof_level(K) == LV) {
-      inv[K] = rsqrt_ftz(team_shfl(diag, K, nl));
+      inv[K] = rsqrtf(team_shfl(diag, K, nl));
       y[K] = team_shfl(b, K, nl) * inv[K];
     }
   }
@@ -334,56 +427,24 @@ struct Dense {
   }
 
   // Assemble, factor and solve (M + diag(arm)) x = b; returns x of this lane's
-  // DOF and 1 / L_kk in idiag.  sw, sv: the lane's motion subspace; the vectors
-  // Ic_b S_b of every DOF are at of.
-  // The columns go in groups whose vectors are all read before the first product
-  // (one at a time, every column waited for its own reads: 54 cycles each).
-  static constexpr int GROUP = 7;
-  template <int B0, int... B>
-  static __device__ __forceinline__ void assemble_group(const SMem& w, int of, V3 sw, V3 sv, const LaneConst& c,
-                                                        int lane, float (&row)[NM], float& diag, iseq<B...>) {
-    float4 f0[sizeof...(B)];
-    float2 f1[sizeof...(B)];
-    ([&] {
-      f0[B] = lds4(w, of + XF * (B0 + B));
-      f1[B] = *reinterpret_cast<const float2*>(&w[of + XF * (B0 + B) + 4]);
-    }(), ...);
-    ([&] {
-      const float p = dot(sw, v3(f0[B].x, f0[B].y, f0[B].z)) + dot(sv, v3(f0[B].w, f1[B].x, f1[B].y));
-      float v = ((c.desc >> (B0 + B)) & 1u) ? p : 0.f;
-      if (B0 + B == lane) { v += c.arm; diag = v; }
-      row[B0 + B] = v;
-    }(), ...);
+  // DOF and 1 / L_kk in idiag.  sw, sv: the lane's motion subspace; fn, ff: Ic S of
+  // its DOF, which every lane's row needs (the vectors at of).
+  static __device__ __forceinline__ void put_vector(const SMem& w, int of, int lane, V3 sw, V3 sv, V3 fn, V3 ff) {
+    sts4(w, of + XF * lane, fn.x, fn.y, fn.z, ff.x);
+    *reinterpret_cast<float2*>(&w[of + XF * lane + 4]) = make_float2(ff.y, ff.z);
   }
-  template <int B0 = 0>
-  static __device__ __forceinline__ void assemble(const SMem& w, int of, V3 sw, V3 sv, const LaneConst& c, int lane,
-                                                  float (&row)[NM], float& diag) {
-    if constexpr (B0 < NM) {
-      assemble_group<B0>(w, of, sw, sv, c, lane, row, diag, make_iseq<(NM - B0 < GROUP ? NM - B0 : GROUP)>{});
-      assemble<B0 + GROUP>(w, of, sw, sv, c, lane, row, diag);
-    }
-  }
-  static __device__ __forceinline__ float solve(const SMem& w, float* fac, int rs, int of, int ol, V3 sw, V3 sv,
-                                                float b, const LaneConst& c, int lane, int nl, float& idiag) {
+  static __device__ __forceinline__ float solve(const SMem& w, float* fac, int rs, int of, int ol, V3 sw, V3 sv, V3 fn,
+                                                V3 ff, float b, const LaneConst& c, int lane, int nl, float& idiag) {
     float row[NM], diag = 1.f;
-    assemble(w, of, sw, sv, c, lane, row, diag);
+    Rows::assemble(w, of, sw, sv, c, lane, row, diag);
     factor(w, ol, row, diag, idiag, b, lane, nl, make_iseq<NM>{});
     team_sync(nl);
     float ls[NM];
     load_row(w, ol, idiag, lane, ls);
-    if (fac && c.own) store_row(fac, rs, ls, lane);
+    if (fac && c.own) Rows::store_row(fac, rs, ls, lane);
     float z = b * idiag;
     back(z, ls, nl, make_iseq<NM>{});
     return z;
-  }
-  // The record keeps the unit factor: row k holds L_kj / L_kk for j < k, next to
-  // 1 / L_kk; 16 bytes of every row side by side.
-  static __device__ __forceinline__ void store_row(float* fac, int rs, const float (&ls)[NM], int lane) {
-#pragma unroll
-    for (int k = 0; k < (NM + 3) / 4; ++k)
-      stg4(fac + 4 * (k * rs + lane), ls[4 * k], 4 * k + 1 < NM ? ls[4 * k + 1 < NM ? 4 * k + 1 : 0] : 0.f,
-           4 * k + 2 < NM ? ls[4 * k + 2 < NM ? 4 * k + 2 : 0] : 0.f,
-           4 * k + 3 < NM ? ls[4 * k + 3 < NM ? 4 * k + 3 : 0] : 0.f);
   }
   // x = (L^T L)^{-1} b from the record: b_a -= (L_ka / L_kk) b_k leaves first,
   // scaled by 1 / L_kk^2, then back as above.
@@ -405,27 +466,112 @@ struct Dense {
   static __device__ __forceinline__ float solve_record(const SMem& w, int of, int rs, int n, float idiag, float b,
                                                        int lane, int nl, iseq<LV...>) {
     float y[NM], lc[NM], ls[NM];
-    const int oc = of + 4 * (lane >> 2) * rs + (lane & 3);
-#pragma unroll
-    for (int k = 0; k < NM; ++k) {
-      const bool use = lane < k && k < n;
-      const float v = w[use ? oc + 4 * k : of];
-      lc[k] = use ? v : 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < (NM + 3) / 4; ++k) {
-      const float4 v = lds4(w, of + 4 * (k * rs + (lane < n ? lane : 0)));
-      const float t[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (4 * k + j < NM) ls[4 * k + j < NM ? 4 * k + j : 0] = lane < n ? t[j] : 0.f;
-    }
+    Rows::load_record(w, of, rs, n, lane, lc, ls);
     (fwd_level<NM - 1 - LV>(b, y, lc, nl, make_iseq<NM>{}), ...);
     float z = b * (idiag * idiag);
     back(z, ls, nl, make_iseq<NM>{});
     return z;
   }
 };
+#else
+// The generic build eliminates root first, M = L L^T, one DOF at a time, with the
+// general kernels' operations in their order (dense_substep): a model's states then
+// do not depend on which of the two forms its batch takes, to the last bit, and no
+// contact, friction or limit switch of a window falls differently in them.  With the
+// tree known at run time only, leaves first would take as many steps.
+//
+// Lane a holds row[b] = M_ab for its ancestors b <= a, its diagonal in diag and the
+// right-hand side in b.  Eliminating DOF k: L_ik = M_ik / L_kk on the lanes i > k,
+// M_ij -= L_ik L_jk, and the forward substitution y_k = b_k / L_kk, b_i -= L_ik y_k in
+// the same pass.  Column k goes to shared memory, where lane k reads it for the
+// backward substitution; the record keeps the rows, next to 1 / L_kk.
+template <int NM>
+struct Dense : DenseRows<NM> {
+  using Rows = DenseRows<NM>;
+  static constexpr int ST = Rows::ST;
+  template <int K, int... J>
+  static __device__ __forceinline__ void trailing(float (&row)[NM], float lk, int nl, iseq<J...>) {
+    ((row[K + 1 + J] = fmaf(-lk, team_shfl(lk, K + 1 + J, nl), row[K + 1 + J])), ...);
+  }
+  template <int K>
+  static __device__ __forceinline__ void column(const SMem& w, int ol, float (&row)[NM], float& diag, float& idiag,
+                                                float& b, int lane, int nl) {
+    const float inv = rsqrtf(team_shfl(diag, K, nl));
+    const float yk = team_shfl(b, K, nl) * inv;
+    const float lk = row[K] * inv;
+    row[K] = lk;
+    if (lane == K) { idiag = inv; b = yk; }
+    if (lane > K) {
+      diag = fmaf(-lk, lk, diag);
+      b = fmaf(-lk, yk, b);
+    }
+    trailing<K>(row, lk, nl, make_iseq<NM - K - 1>{});
+  }
+  template <int... K>
+  static __device__ __forceinline__ void factor(const SMem& w, int ol, float (&row)[NM], float& diag, float& idiag,
+                                                float& b, int lane, int nl, iseq<K...>) {
+    (column<K>(w, ol, row, diag, idiag, b, lane, nl), ...);
+  }
+  // L^T x = y: x_k = y_k / L_kk, y_a -= L_ka x_k, the last DOF first; lc: this lane's
+  // column of L.
+  template <int K>
+  static __device__ __forceinline__ void back_step(float& b, const float (&lc)[NM], float idiag, int lane, int nl) {
+    const float xk = team_shfl(b * idiag, K, nl);
+    b = lane == K ? xk : fmaf(-lc[K], xk, b);
+  }
+  template <int... K>
+  static __device__ __forceinline__ void back(float& b, const float (&lc)[NM], float idiag, int lane, int nl, iseq<K...>) {
+    (back_step<NM - 1 - K>(b, lc, idiag, lane, nl), ...);
+  }
+  // Assemble, factor and solve (M + diag(arm)) x = b; returns x of this lane's
+  // DOF and 1 / L_kk in idiag.  sw, sv: the lane's motion subspace, which every lane's
+  // row needs (the vectors at of); fn, ff: Ic S of its DOF.
+  static __device__ __forceinline__ void put_vector(const SMem& w, int of, int lane, V3 sw, V3 sv, V3 fn, V3 ff) {
+    sts4(w, of + XF * lane, sw.x, sw.y, sw.z, sv.x);
+    *reinterpret_cast<float2*>(&w[of + XF * lane + 4]) = make_float2(sv.y, sv.z);
+  }
+  static __device__ __forceinline__ float solve(const SMem& w, float* fac, int rs, int of, int ol, V3 sw, V3 sv, V3 fn,
+                                                V3 ff, float b, const LaneConst& c, int lane, int nl, float& idiag) {
+    float row[NM], diag = 1.f;
+    Rows::assemble(w, of, fn, ff, c, lane, row, diag);
+    factor(w, ol, row, diag, idiag, b, lane, nl, make_iseq<NM>{});
+#pragma unroll
+    for (int k = 0; k < NM; ++k) row[k] = k < lane ? row[k] : 0.f;
+    if (lane < NM) {
+#pragma unroll
+      for (int k = 0; k < (NM + 3) / 4; ++k)
+        sts4(w, ol + ST * lane + 4 * k, row[4 * k], 4 * k + 1 < NM ? row[4 * k + 1 < NM ? 4 * k + 1 : 0] : 0.f,
+             4 * k + 2 < NM ? row[4 * k + 2 < NM ? 4 * k + 2 : 0] : 0.f,
+             4 * k + 3 < NM ? row[4 * k + 3 < NM ? 4 * k + 3 : 0] : 0.f);
+    }
+    if (fac && c.own) Rows::store_row(fac, rs, row, lane);
+    team_sync(nl);
+    float lc[NM];
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {   // zero in the row's own upper part
+      const float v = w[ol + ST * k + (lane < NM ? lane : 0)];
+      lc[k] = lane < k ? v : 0.f;
+    }
+    back(b, lc, idiag, lane, nl, make_iseq<NM>{});
+    return b;
+  }
+  // x = (L L^T)^{-1} b from the record
+  template <int K>
+  static __device__ __forceinline__ void fwd_step(float& b, const float (&ls)[NM], float idiag, int lane, int nl) {
+    const float yk = team_shfl(b * idiag, K, nl);
+    b = lane == K ? yk : fmaf(-ls[K], yk, b);
+  }
+  template <int... K>
+  static __device__ __forceinline__ float solve_record(const SMem& w, int of, int rs, int n, float idiag, float b,
+                                                       int lane, int nl, iseq<K...>) {
+    float lc[NM], ls[NM];
+    Rows::load_record(w, of, rs, n, lane, lc, ls);
+    (fwd_step<K>(b, ls, idiag, lane, nl), ...);
+    back(b, lc, idiag, lane, nl, iseq<K...>{});
+    return b;
+  }
+};
+#endif
 
 // Position update of the free root (replicated on every lane) from its new
 // velocity: p += h R v, quat <- normalise(quat + h/2 quat (x) (w, 0)); see
@@ -452,10 +598,14 @@ struct LaneLink {
   float si[10];         // m, h, Io
   V3 wn, wf, fn, ff;
 };
+// COMPOSITE: the composite inertia's product with a motion subspace, whose y component
+// rounds as the general kernels' (si_mul of shac_device.cuh).
+template <bool COMPOSITE = false>
 __device__ __forceinline__ void si_mul(const float (&si)[10], V3 xw, V3 xv, V3& yn, V3& yf) {
   const V3 h = v3(si[1], si[2], si[3]);
-  yn = v3(si[4] * xw.x + si[7] * xw.y + si[8] * xw.z, si[7] * xw.x + si[5] * xw.y + si[9] * xw.z,
-          si[8] * xw.x + si[9] * xw.y + si[6] * xw.z) + cross(h, xv);
+  yn = v3(sum3(si[4], xw.x, si[7], xw.y, si[8], xw.z),
+          COMPOSITE ? sum3(si[5], xw.y, si[7], xw.x, si[9], xw.z) : sum3(si[7], xw.x, si[5], xw.y, si[9], xw.z),
+          sum3(si[8], xw.x, si[9], xw.y, si[6], xw.z)) + cross(h, xv);
   yf = si[0] * xv - cross(h, xw);
 }
 __device__ __forceinline__ void lane_local(const DevModel& M, const SMem& w, const LaneConst& c, float zroot,
@@ -465,12 +615,7 @@ __device__ __forceinline__ void lane_local(const DevModel& M, const SMem& w, con
   Ic.m[0] = c.icom[0]; Ic.m[4] = c.icom[1]; Ic.m[8] = c.icom[2];
   Ic.m[1] = Ic.m[3] = c.icom[3]; Ic.m[2] = Ic.m[6] = c.icom[4]; Ic.m[5] = Ic.m[7] = c.icom[5];
   const M33 Iw = mulBT(mul(k.R, Ic), k.R);
-  const float cc = dot(cm, cm), m = c.mass;
-  const V3 h = m * cm;
-  k.si[0] = m; k.si[1] = h.x; k.si[2] = h.y; k.si[3] = h.z;
-  k.si[4] = Iw.m[0] + m * (cc - cm.x * cm.x); k.si[5] = Iw.m[4] + m * (cc - cm.y * cm.y);
-  k.si[6] = Iw.m[8] + m * (cc - cm.z * cm.z); k.si[7] = Iw.m[1] - m * cm.x * cm.y;
-  k.si[8] = Iw.m[2] - m * cm.x * cm.z; k.si[9] = Iw.m[5] - m * cm.y * cm.z;
+  spatial_inertia(Iw, c.mass, cm, k.si);
   k.wn = k.wf = v3(0.f, 0.f, 0.f);
   V3 xl = c.cpos;
   float rad = c.crad;
@@ -482,10 +627,9 @@ __device__ __forceinline__ void lane_local(const DevModel& M, const SMem& w, con
     if (d < 0.f) {
       const V3 vp = k.Vv + cross(k.Vw, x);
       const float fn = (-M.ke + M.kd * vp.z) * d;
-      const float v2 = vp.x * vp.x + vp.y * vp.y;
-      const float iv = v2 > MIN_NORMAL ? rsqrt_refined(v2) : 0.f;   // 1 / |v_t|
+      const float vt = sqrtf(sum2(vp.x, vp.x, vp.y, vp.y));
       const float fmax = M.mu * fabsf(fn);
-      const float sc = M.kt * (v2 * iv) <= fmax ? M.kt : fmax * iv;
+      const float sc = M.kt * vt <= fmax ? M.kt : fmax / vt;
       f.x = -sc * vp.x; f.y = -sc * vp.y;
       f.z = fn;
     }
@@ -669,9 +813,6 @@ __device__ __forceinline__ void lane_substep(const DevModel& M, const SMem& w, c
   const bool root = M.root_free && lane == 0;
   LaneLink k;
   M33 R0;                                   // the free root's rotation, on every lane
-  V3 wl = v3(0.f, 0.f, 0.f), vl = wl;
-  if (c.jt == J_REV) wl = s.qd * c.axis;
-  if (c.jt == J_PRIS) vl = s.qd * c.axis;
   k.R = mul(c.jrot, axis_angle(c.axis, c.jt == J_REV ? s.q : 0.f));
   k.P = c.jpos;
   if (c.jt == J_PRIS) k.P = k.P + s.q * mul(k.R, c.axis);
@@ -680,41 +821,57 @@ __device__ __forceinline__ void lane_substep(const DevModel& M, const SMem& w, c
     if (root) {
       k.R = R0;
       k.P = v3(0.f, 0.f, 0.f);
-      wl = v3(s.rqd[0], s.rqd[1], s.rqd[2]);
-      vl = v3(s.rqd[3], s.rqd[4], s.rqd[5]);
     }
   }
-  // world pose: T_i = T_anc T_i, the ancestor twice as far in every round
+  // world pose: T_i = T_anc T_i, the ancestor twice as far in every round, or the
+  // parent, a level in every round (path_sums)
+#ifdef SHAC_SPEC_ANC
 #pragma unroll
   for (int r = 0; r < M.nround; ++r) {
     const unsigned a = (c.anc >> (6 * r)) & 63u;
+    const int src = (int)(a & 31u);
+    const bool take = a < 32u;
+#else
+  const int src = (int)(c.anc & 31u);
+  for (int r = 1; r <= M.deepest; ++r) {
+    const bool take = c.depth == r;
+#endif
     M33 Rp;
 #pragma unroll
-    for (int j = 0; j < 9; ++j) Rp.m[j] = team_shfl(k.R.m[j], (int)(a & 31u), nl);
-    const V3 Pp = team_shfl(k.P, (int)(a & 31u), nl);
-    if (a < 32u) {
+    for (int j = 0; j < 9; ++j) Rp.m[j] = team_shfl(k.R.m[j], src, nl);
+    const V3 Pp = team_shfl(k.P, src, nl);
+    if (take) {
       k.P = Pp + mul(Rp, k.P);
       k.R = mul(Rp, k.R);
     }
   }
-  // joint velocity, motion subspace, velocities and accelerations (qdd = 0)
+  // motion subspace, joint velocity, velocities and accelerations (qdd = 0)
   const V3 ax = mul(k.R, c.axis);
-  const V3 uw = mul(k.R, wl);
-  const V3 uv = cross(k.P, uw) + mul(k.R, vl);
+  V3 sw = c.jt == J_REV ? ax : v3(0.f, 0.f, 0.f);
+  V3 sv = c.jt == J_REV ? cross(k.P, ax) : (c.jt == J_PRIS ? ax : v3(0.f, 0.f, 0.f));
+  V3 uw = s.qd * sw, uv = s.qd * sv;
+  if (M.root_free) {
+    if (root) {
+      uw = uv = v3(0.f, 0.f, 0.f);          // a DOF at a time, as lk_subspace_vel
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        uw = uw + s.rqd[j] * col(R0, j);
+        uv = uv + s.rqd[3 + j] * col(R0, j);
+      }
+    }
+    if (lane < 6) {                         // the root's columns (its origin is the reference point)
+      const int d = lane % 3;
+      const V3 e = d == 0 ? col(R0, 0) : (d == 1 ? col(R0, 1) : col(R0, 2));
+      sw = lane < 3 ? e : v3(0.f, 0.f, 0.f);
+      sv = lane < 3 ? v3(0.f, 0.f, 0.f) : e;
+    }
+  }
   k.Vw = uw; k.Vv = uv;
-  path_sums(M, c.anc, nl, k.Vw, k.Vv);
+  path_sums(M, c, nl, k.Vw, k.Vv);
   k.aw = cross(k.Vw, uw);
   k.av = cross(k.Vw, uv) + cross(k.Vv, uw);
   k.av = k.av + c.base;
-  path_sums(M, c.anc, nl, k.aw, k.av);
-  V3 sw = c.jt == J_REV ? ax : v3(0.f, 0.f, 0.f);
-  V3 sv = c.jt == J_REV ? cross(k.P, ax) : (c.jt == J_PRIS ? ax : v3(0.f, 0.f, 0.f));
-  if (M.root_free && lane < 6) {            // the root's columns (its origin is the reference point)
-    const int d = lane % 3;
-    const V3 e = d == 0 ? col(R0, 0) : (d == 1 ? col(R0, 1) : col(R0, 2));
-    sw = lane < 3 ? e : v3(0.f, 0.f, 0.f);
-    sv = lane < 3 ? v3(0.f, 0.f, 0.f) : e;
-  }
+  path_sums(M, c, nl, k.aw, k.av);
   lane_local(M, w, c, M.root_free ? s.rq[2] : 0.f, k);
   const bool link = c.link >= 0;
   if (M.nseg > 0) {   // muscles: a segment spans two links, so the poses go through memory
@@ -760,14 +917,11 @@ __device__ __forceinline__ void lane_substep(const DevModel& M, const SMem& w, c
   lane_sums(M, w, x, c, link, lane, nl);
   // right-hand side and the vectors Ic S
   float b = 0.f;
+  V3 fn, ff;
   {
     const float ic[10] = {x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7], x[8], x[9]};
-    V3 fn, ff;
-    si_mul(ic, sw, sv, fn, ff);
-    if (lane < nm) {
-      sts4(w, of + XF * lane, fn.x, fn.y, fn.z, ff.x);
-      *reinterpret_cast<float2*>(&w[of + XF * lane + 4]) = make_float2(ff.y, ff.z);
-    }
+    si_mul<true>(ic, sw, sv, fn, ff);
+    if (lane < nm) Dense<2>::put_vector(w, of, lane, sw, sv, fn, ff);
     if (c.own) {
       float t = tau0;
       if (c.jt == J_REV || c.jt == J_PRIS) {
@@ -781,7 +935,7 @@ __device__ __forceinline__ void lane_substep(const DevModel& M, const SMem& w, c
   float idiag = 1.f, qdd = 0.f;
   const int ol = of + XF * nm;
   switch (nm) {
-#define SHAC_CASE(N) case N: qdd = Dense<N>::solve(w, rec ? rec + ro.fac : nullptr, ro.rs, of, ol, sw, sv, b, c, lane, nl, idiag); break;
+#define SHAC_CASE(N) case N: qdd = Dense<N>::solve(w, rec ? rec + ro.fac : nullptr, ro.rs, of, ol, sw, sv, fn, ff, b, c, lane, nl, idiag); break;
     SHAC_DENSE_CASES(SHAC_CASE)
 #undef SHAC_CASE
     default: break;
@@ -849,7 +1003,7 @@ struct LaneBars {
   float rqb[7];
 };
 
-// x_i += x_anc for two pairs of vectors at once (path_sums).
+// Sums of four vectors along the path to the root (own value included), by doubling.
 __device__ __forceinline__ void path_sums2(const DevModel& M, unsigned anc, int nl, V3& a, V3& b, V3& c, V3& d) {
 #pragma unroll
   for (int r = 0; r < M.nround; ++r) {
