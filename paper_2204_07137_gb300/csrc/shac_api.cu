@@ -137,7 +137,8 @@ static void compute_muscle_slots(shac_model* m) {
 
 // Lane columns of the model (shac_team.cuh): lane d owns DOF d, and the link
 // whose first DOF it is; links without a DOF take the lanes from nv on.  More
-// than 32 lanes needed: the model has no lane form.
+// than 32 lanes needed, or a link with more contacts than its record holds
+// switches for: the model has no lane form.
 static void compute_lanes(shac_model* m) {
   const int L = m->L, nv = m->nv;
   std::vector<int> lane_of(L), level(L, 0);
@@ -147,6 +148,8 @@ static void compute_lanes(shac_model* m) {
     if (m->parent[i] >= 0) level[i] = level[m->parent[i]] + 1;
     deepest = std::max(deepest, level[i]);
   }
+  for (int i = 0; i < L; ++i)
+    if (m->lc_ptr[i + 1] - m->lc_ptr[i] > LINK_CONTACTS) next = LANE_COLS + 1;
   m->lanes_needed = next;
   compute_muscle_slots(m);
   m->nround = 0;

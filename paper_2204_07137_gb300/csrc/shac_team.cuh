@@ -50,8 +50,8 @@ constexpr int MASS_COLS = LI_DESC;
 #else
 constexpr int MASS_COLS = LI_ROW;
 #endif
-constexpr float MIN_NORMAL = 1.17549435e-38f;
 constexpr int MSLOTS = 32;   // columns of the muscles' via-point items
+constexpr int LINK_CONTACTS = 16;   // contacts of a link whose switches one record word holds
 
 struct LaneConst {
   int link, jt, qi, act, c0, c1, dlink, depth, ms0, ms1;
@@ -161,7 +161,8 @@ __host__ __device__ constexpr int lane_xchg_floats(int L, int nm) {
 // What the reverse pass reads, one block per substep (offsets in floats, every
 // array of 16-byte elements indexed by link or DOF, so that lanes read and
 // write consecutive 16 bytes):
-//   8 float4 [link]: R, P, spatial inertia, velocity, external wrench (32 of 34)
+//   8 float4 [link]: R, P, spatial inertia, velocity, external wrench (32 of 34); in the
+//                    place of the inertia's mass, a model constant, the contacts' switches
 //   1 float4 [DOF]:  qd, qdd, 1 / L_kk, q (one-DOF joints)
 //   rows of the unit factor, float4 [entry / 4][DOF]
 //   free root: q 7, qd 6, qdd 6, pad
@@ -597,6 +598,11 @@ struct LaneLink {
   V3 P, Vw, Vv, aw, av;
   float si[10];         // m, h, Io
   V3 wn, wf, fn, ff;
+  // two bits a contact, the link's first lowest: touching, and sliding slowly (the
+  // viscous branch).  The reverse pass takes the branches the forward took from here: a
+  // test repeated from the record, within rounding of its switch, could fall the other
+  // way and give the gradient of another force than the one that acted.
+  unsigned contacts;
 };
 // COMPOSITE: the composite inertia's product with a motion subspace, whose y component
 // rounds as the general kernels' (si_mul of shac_device.cuh).
@@ -617,6 +623,7 @@ __device__ __forceinline__ void lane_local(const DevModel& M, const SMem& w, con
   const M33 Iw = mulBT(mul(k.R, Ic), k.R);
   spatial_inertia(Iw, c.mass, cm, k.si);
   k.wn = k.wf = v3(0.f, 0.f, 0.f);
+  k.contacts = 0u;
   V3 xl = c.cpos;
   float rad = c.crad;
   for (int e = c.c0; e < c.c1;) {   // contact spheres (the model of lk_local)
@@ -629,7 +636,9 @@ __device__ __forceinline__ void lane_local(const DevModel& M, const SMem& w, con
       const float fn = (-M.ke + M.kd * vp.z) * d;
       const float vt = sqrtf(sum2(vp.x, vp.x, vp.y, vp.y));
       const float fmax = M.mu * fabsf(fn);
-      const float sc = M.kt * vt <= fmax ? M.kt : fmax / vt;
+      const bool slow = M.kt * vt <= fmax;
+      const float sc = slow ? M.kt : fmax / vt;
+      k.contacts |= (slow ? 3u : 1u) << (2 * (e - c.c0));
       f.x = -sc * vp.x; f.y = -sc * vp.y;
       f.z = fn;
     }
@@ -900,7 +909,7 @@ __device__ __forceinline__ void lane_substep(const DevModel& M, const SMem& w, c
     stg4(r, k.R.m[0], k.R.m[1], k.R.m[2], k.R.m[3]);
     stg4(r + fs, k.R.m[4], k.R.m[5], k.R.m[6], k.R.m[7]);
     stg4(r + 2 * fs, k.R.m[8], k.P.x, k.P.y, k.P.z);
-    stg4(r + 3 * fs, k.si[0], k.si[1], k.si[2], k.si[3]);
+    stg4(r + 3 * fs, __uint_as_float(k.contacts), k.si[1], k.si[2], k.si[3]);
     stg4(r + 4 * fs, k.si[4], k.si[5], k.si[6], k.si[7]);
     stg4(r + 5 * fs, k.si[8], k.si[9], k.Vw.x, k.Vw.y);
     stg4(r + 6 * fs, k.Vw.z, k.Vv.x, k.Vv.y, k.Vv.z);
@@ -1039,7 +1048,7 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
     k.R.m[0] = a0.x; k.R.m[1] = a0.y; k.R.m[2] = a0.z; k.R.m[3] = a0.w;
     k.R.m[4] = a1.x; k.R.m[5] = a1.y; k.R.m[6] = a1.z; k.R.m[7] = a1.w;
     k.R.m[8] = a2.x; k.P = v3(a2.y, a2.z, a2.w);
-    k.si[0] = a3.x; k.si[1] = a3.y; k.si[2] = a3.z; k.si[3] = a3.w;
+    k.contacts = __float_as_uint(a3.x); k.si[0] = c.mass; k.si[1] = a3.y; k.si[2] = a3.z; k.si[3] = a3.w;
     k.si[4] = a4.x; k.si[5] = a4.y; k.si[6] = a4.z; k.si[7] = a4.w;
     k.si[8] = a5.x; k.si[9] = a5.y; k.Vw = v3(a5.z, a5.w, a6.x); k.Vv = v3(a6.y, a6.z, a6.w);
     k.wn = v3(a7.x, a7.y, a7.z); k.wf = v3(a7.w, a8.x, a8.y);
@@ -1178,21 +1187,21 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
   V3 xl = c.cpos;
   float rad = c.crad;
   for (int e = c.c0; e < c.c1;) {
-    V3 x = k.P + mul(k.R, xl);
-    x.z -= rad;
-    const float dep = x.z + zroot;
-    if (dep < 0.f) {
+    const unsigned on = k.contacts >> (2 * (e - c.c0));
+    if (on & 1u) {
+      V3 x = k.P + mul(k.R, xl);
+      x.z -= rad;
+      const float dep = x.z + zroot;
       const V3 vp = k.Vv + cross(k.Vw, x);
       const float fn = (-M.ke + M.kd * vp.z) * dep;
-      const float v2 = vp.x * vp.x + vp.y * vp.y;
-      const float iv = v2 > MIN_NORMAL ? rsqrt_refined(v2) : 0.f;   // 1 / |v_t|
+      const bool slow = (on & 2u) != 0u;
+      const float iv = slow ? 0.f : 1.f / sqrtf(sum2(vp.x, vp.x, vp.y, vp.y));   // 1 / |v_t|
       const float fmax = M.mu * fabsf(fn);
       const V3 neb = -nb;
       const V3 fbar = cross(neb, x) - fb;
       float fnb = fbar.z;
       V3 f, vpb = v3(0.f, 0.f, 0.f);
       f.z = fn;
-      const bool slow = M.kt * (v2 * iv) <= fmax;
       const float sc = slow ? M.kt : fmax * iv;
       f.x = -sc * vp.x; f.y = -sc * vp.y;
       vpb.x = -sc * fbar.x;

@@ -93,3 +93,57 @@ def test_gradients_do_not_depend_on_the_form(seed):
     a, b = (np.concatenate(_window(m, N, 2, seed, form)[2:]).astype(np.float64) for form in (True, False))
     err = np.linalg.norm(a - b, axis=0) / np.linalg.norm(b, axis=0)
     assert err.max() < 1e-3, (int(err.argmax()), float(err.max()))
+
+
+def sliding_ball(contacts=1):
+    b = I._Builder("ball")
+    root = b.link(-1, I.FREE, mass=1.0, com=(0, 0, 0), inertia=0.01 * np.eye(3))
+    for k in range(contacts):
+        b.contact(root, (0, 0, 0), 0.1 if k == contacts - 1 else 0.05 + 0.002 * k)
+    return b.finish(act_dof=[4], act_gear=[1.0], dt=I.CONTROL_DT, substeps=1, ke=5e3, kd=100.0, kt=20.0, mu=0.5, root_z=0.099)
+
+
+@pytest.mark.parametrize("contacts", [1, 16, 17])
+@pytest.mark.parametrize("switch", ["slip", "touch"])
+def test_reverse_takes_the_contact_branch_of_the_forward(switch, contacts):
+    """Balls whose sliding speed (or height) steps through its switch a few units in
+    the last place at a time, at 64 depths (speeds), vertical speeds and directions.
+    The gradient is the one of the branch the force took: the general kernels', which
+    keep the forward's depth and force (their branch differs from the other's by
+    h kt / m = 0.3 of a unit cotangent; rounding by less than 1e-5).  A link of 16 contacts
+    fills a record's word, one of 17 has the general kernels on both sides."""
+    from paper_2204_07137_gb300.sim import Simulator
+    m, n, steps = sliding_ball(contacts), 64, 129
+    rng = np.random.default_rng(2)
+    N = n * steps
+    depth = np.repeat(rng.uniform(1e-4, 3e-3, n), steps)
+    vz = np.repeat(rng.uniform(-0.5, 0.5, n), steps)
+    phi = np.repeat(rng.uniform(0, 2 * np.pi, n), steps)
+    ulp = np.tile(np.arange(steps) - steps // 2, n) * 2.0 ** -24
+    speed = np.repeat(rng.uniform(0.05, 1.0, n), steps)
+    if switch == "slip":   # kt v = mu |fn|
+        speed = 0.5 * np.abs((-5e3 + 100 * vz) * depth) / 20 * (1 + 4 * ulp)
+    else:
+        depth = 0.1 * ulp / 16
+    q, qd = np.zeros((7, N)), np.zeros((6, N))
+    q[2], q[6] = 0.1 - depth, 1.0
+    if switch == "touch":  # the contact's height is the root's less the radius: exact steps about zero
+        q[2] = np.float32(0.1) + 0.1 * ulp
+    qd[3], qd[4], qd[5] = speed * np.cos(phi), speed * np.sin(phi), vz
+    out = []
+    for lane_form in (True, False):
+        sim = Simulator([(m, N)] + ([] if lane_form else [(many_links(), 1)]), form="batched", h_max=1)
+        pad = lambda x: torch.cat([T(x)] + ([] if lane_form else [torch.zeros(1, device="cuda")]))  # noqa: E731
+        x = [pad(q), pad(qd), pad(np.zeros((1, N)))]
+        y = sim.step(*x)
+        g = sim.step_adjoint(*x, torch.zeros_like(y[0]), torch.ones_like(y[1]), torch.zeros_like(y[2]))
+        torch.cuda.synchronize()
+        out.append([v[:k * N].cpu().numpy().reshape(k, N) for v, k in ((y[0], 7), (y[1], 6), (g[0], 7), (g[1], 6))])
+    for a, b in zip(out[0][:2], out[1][:2]):
+        np.testing.assert_array_equal(a, b)
+    # both branches are taken: the sliding's show in the gradients of the horizontal
+    # velocities, the contact's in that of the height
+    both = out[1][3][3:5] if switch == "slip" else out[1][2][2:3]
+    assert len({tuple(v) for v in np.round(both.T, 1)}) > 1
+    for a, b in zip(out[0][2:], out[1][2:]):
+        np.testing.assert_allclose(a, b, rtol=1e-3, atol=1e-3 * np.abs(b).max())
