@@ -21,7 +21,7 @@ struct shac_model {
   int height_q = -1, vx_dof = -1;   // reward / termination coordinates (free root: 2 / world vx)
   std::vector<int> parent, jtype, qs, ds, nd, lvl_ptr, lvl_link, ch_ptr, ch_idx, lc_ptr, lc_idx, lm_ptr, lm_idx, dof_link,
       dof_k,
-      dof_act, item_link, seg_mus, mus_seg_ptr, anc_mask, chain_tail, ln_i, ms_ptr, sg_place;
+      dof_act, item_link, seg_mus, mus_seg_ptr, anc_mask, chain_tail, on_root, ln_i, ms_ptr, sg_place;
   std::vector<float> axis, jpos, jrot, mass, com, icom, qlo, qhi, arm, damp, gear, item_pos, crad, fmax, rwq, rwqd, ln_f, sg_f;
   int lanes_needed = 0, nround = 0, deepest = 0, mrows = 0;
   DevModel layout, lane_layout;   // sizes + scratch offsets (pointers unset): general and lane form
@@ -170,6 +170,7 @@ static void compute_lanes(shac_model* m) {
     I(LI_LINK, l) = i; I(LI_JT, l) = m->jtype[i]; I(LI_Q, l) = m->qs[i];
     I(LI_C0, l) = m->lc_ptr[i]; I(LI_C1, l) = m->lc_ptr[i + 1];
     I(LI_DEPTH, l) = level[i];
+    I(LI_ON_ROOT, l) = m->on_root[i];
     unsigned anc = 0;                     // the 2^r-th ancestors' lanes, 6 bits each (63: none)
     for (int r = 0; r < 5; ++r) {
       int j = i;
@@ -321,6 +322,8 @@ extern "C" shac_status shac_model_create(const shac_model_desc* dsc, shac_model*
     for (int k = 0; k < 3; ++k) m->com.push_back(dsc->com[3 * i + k]);
     for (int k = 0; k < 6; ++k) m->icom.push_back(dsc->inertia[6 * i + k]);
   }
+  for (int i = 0; i < L; ++i)
+    m->on_root.push_back(m->parent[i] < 0 ? (i == 0 && m->root_free) : m->on_root[m->parent[i]]);
   // children lists
   m->ch_ptr.assign(L + 1, 0);
   for (int i = 0; i < L; ++i) {
@@ -469,6 +472,7 @@ static shac_status upload_model(const shac_model* m, Group& g) {
   addi(&d.parent, m->parent); addi(&d.jtype, m->jtype); addi(&d.qs, m->qs); addi(&d.ds, m->ds); addi(&d.nd, m->nd);
   addi(&d.lvl_ptr, m->lvl_ptr); addi(&d.lvl_link, m->lvl_link); addi(&d.chain_tail, m->chain_tail); addi(&d.ch_ptr, m->ch_ptr); addi(&d.ch_idx, m->ch_idx);
   addi(&d.lc_ptr, m->lc_ptr); addi(&d.lc_idx, m->lc_idx); addi(&d.lm_ptr, m->lm_ptr); addi(&d.lm_idx, m->lm_idx);
+  addi(&d.on_root, m->on_root);
   addi(&d.dof_link, m->dof_link); addi(&d.dof_k, m->dof_k);
   addi(&d.dof_act, m->dof_act); addi(&d.item_link, m->item_link); addi(&d.seg_mus, m->seg_mus);
   addi(&d.mus_seg_ptr, m->mus_seg_ptr);

@@ -82,6 +82,7 @@ struct DevModel {
   const int *ch_ptr, *ch_idx;            // children lists
   const int *lc_ptr, *lc_idx;            // contact items attached to each link
   const int *lm_ptr, *lm_idx;            // muscle via-point items attached to each link
+  const int* on_root;                    // 1: a link of the free root's tree (positions relative to the root origin)
   const float *axis, *jpos, *jrot, *mass, *com, *icom;
   // dofs
   const int *dof_link, *dof_k, *dof_act;
@@ -623,7 +624,7 @@ __device__ __forceinline__ void lk_local(const DevModel& M, const Mem& w, int i)
   V3 wn = v3(0.f, 0.f, 0.f), wf = v3(0.f, 0.f, 0.f);
   const int k0 = __ldg(M.lc_ptr + i), k1 = __ldg(M.lc_ptr + i + 1);
   if (k0 != k1) {
-    const float zroot = M.root_free ? w[M.o_Q + 2] : 0.f;
+    const float zroot = __ldg(M.on_root + i) ? w[M.o_Q + 2] : 0.f;
     for (int k = k0; k < k1; ++k) {
       const int ci = __ldg(M.lc_idx + k);
       V3 x = P + mul(R, cld3(M.item_pos + 3 * ci));
@@ -1454,7 +1455,7 @@ __device__ __forceinline__ void lk_adj_local(const DevModel& M, const Mem& w, in
         vpb.x += vtb * vp.x / vt;
         vpb.y += vtb * vp.y / vt;
       }
-      // fn = (-ke + kd ddot) d, d = x.z + root height
+      // fn = (-ke + kd ddot) d, d = x.z + root height (in the free root's tree)
       db = fnb * (-M.ke + M.kd * vp.z);
       xb.z += db;
       vpb.z += fnb * M.kd * dep;
@@ -1464,7 +1465,7 @@ __device__ __forceinline__ void lk_adj_local(const DevModel& M, const Mem& w, in
       Pb = Pb + xb;
       add_outer(Rb, xb, cld3(M.item_pos + 3 * c));
     }
-    w[M.o_ITB + 10 * c + 9] = db;
+    w[M.o_ITB + 10 * c + 9] = __ldg(M.on_root + i) ? db : 0.f;
   }
   st3(w, lwork(M, i) + LW_VB, vwb);
   st3(w, lwork(M, i) + LW_VB + 3, vvb);
@@ -1733,8 +1734,8 @@ __device__ __forceinline__ void root_dof_terms(const DevModel& M, const Mem& w, 
 
 // q_bar of link i's joint from its final pose cotangents: revolute
 // dR/dq = [a]x R with a = R ax; prismatic dP/dq = a; free root: the
-// quaternion's share through R(quat), and the root height receives every
-// contact depth's cotangent (depth = x.z + root height).
+// quaternion's share through R(quat), and the root height receives the depth
+// cotangent of every contact of its tree (depth = x.z + root height).
 // WORLD: the R_bar slot holds the subtree sum of Q and the P_bar slot that of
 // P_bar (team form); R_bar = (Q - P_bar P^T) R is formed first.
 template <bool WORLD, class Mem>

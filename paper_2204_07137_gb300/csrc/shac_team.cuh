@@ -39,7 +39,7 @@
 namespace shac {
 
 // This lane's share of the model (DevModel::ln_i, ln_f: one column per lane).
-enum { LI_LINK = 0, LI_JT, LI_ANC, LI_Q, LI_ACT, LI_C0, LI_C1, LI_DESC, LI_ROW, LI_DLINK, LI_DEPTH, LI_N };
+enum { LI_LINK = 0, LI_JT, LI_ANC, LI_Q, LI_ACT, LI_C0, LI_C1, LI_DESC, LI_ROW, LI_DLINK, LI_DEPTH, LI_ON_ROOT, LI_N };
 enum { LF_AXIS = 0, LF_JROT = 3, LF_JPOS = 12, LF_COM = 15, LF_ICOM = 18, LF_MASS = 24, LF_ARM, LF_DAMP, LF_GEAR,
        LF_QLO, LF_QHI, LF_CPOS, LF_CRAD = LF_CPOS + 3, LF_BASE, LF_N = LF_BASE + 3 };
 constexpr int LANE_COLS = 32;
@@ -57,6 +57,7 @@ struct LaneConst {
   int link, jt, qi, act, c0, c1, dlink, depth, ms0, ms1;
   unsigned anc, cols;   // cols: entries of the lane's mass-matrix row
   bool own;             // lane < nv
+  bool on_root;         // the link is of the free root's tree
   V3 axis, jpos, com, cpos, base;   // cpos, crad: the link's first contact; base: -g on a root link
   M33 jrot;
   float icom[6];
@@ -76,6 +77,7 @@ __device__ __forceinline__ LaneConst lane_const(const DevModel& M, int lane) {
   c.ms0 = c.ms1 = 0;
   if (M.nseg > 0 && c.link >= 0) { c.ms0 = __ldg(M.ms_ptr + c.link); c.ms1 = __ldg(M.ms_ptr + c.link + 1); }
   c.own = lane < M.nv;
+  c.on_root = gi(LI_ON_ROOT) != 0;
   c.axis = v3(gf(LF_AXIS), gf(LF_AXIS + 1), gf(LF_AXIS + 2));
   c.jpos = v3(gf(LF_JPOS), gf(LF_JPOS + 1), gf(LF_JPOS + 2));
   c.com = v3(gf(LF_COM), gf(LF_COM + 1), gf(LF_COM + 2));
@@ -881,7 +883,7 @@ __device__ __forceinline__ void lane_substep(const DevModel& M, const SMem& w, c
   k.av = cross(k.Vw, uv) + cross(k.Vv, uw);
   k.av = k.av + c.base;
   path_sums(M, c, nl, k.aw, k.av);
-  lane_local(M, w, c, M.root_free ? s.rq[2] : 0.f, k);
+  lane_local(M, w, c, c.on_root ? s.rq[2] : 0.f, k);
   const bool link = c.link >= 0;
   if (M.nseg > 0) {   // muscles: a segment spans two links, so the poses go through memory
     muscle_put_pose(M, w, c.link, k.R, k.P);
@@ -1065,7 +1067,7 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
   if (M.root_free) {
     const int o = M.o_R + ro.root;
     const float4 b0 = lds4(w, o), b1 = lds4(w, o + 4), b2 = lds4(w, o + 8), b3 = lds4(w, o + 12), b4 = lds4(w, o + 16);
-    zroot = b0.z; rx = b0.w; ry = b1.x; rz = b1.y; rw = b1.z;
+    zroot = c.on_root ? b0.z : 0.f; rx = b0.w; ry = b1.x; rz = b1.y; rw = b1.z;
     rqd[0] = b1.w; rqd[1] = b2.x; rqd[2] = b2.y; rqd[3] = b2.z; rqd[4] = b2.w; rqd[5] = b3.x;
     rqdd[0] = b3.y; rqdd[1] = b3.z; rqdd[2] = b3.w; rqdd[3] = b4.x; rqdd[4] = b4.y; rqdd[5] = b4.z;
     R0 = quat_to_R(rx, ry, rz, rw);
