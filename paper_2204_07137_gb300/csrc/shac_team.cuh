@@ -128,19 +128,13 @@ __device__ __forceinline__ void path_sums(const DevModel& M, const LaneConst& c,
 #endif
 }
 
-// 1 / sqrt(x) to 2 ulp, a subnormal x taken as zero: rsqrtf without the scaling
-// that saves subnormal arguments, five instructions on the pivots' chain.
-__device__ __forceinline__ float rsqrt_ftz(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-// 1 / sqrt(x) for a normal x, refined by a Newton step of y -> y (3 - x y^2) / 2 to
-// within an ulp or so: what 1.f / sqrtf(x) gives, without its two special-case
-// branches, which keep the compiler from overlapping neighbouring evaluations.
+// 1 / sqrt(x): rsqrtf (documented maximum error 2 ulp) and one Newton step of
+// y -> y (3 - x y^2) / 2, to a relative error below 1.5 * 2^-24; 0 gives infinity and
+// infinity 0, where the step has no value.  Serves muscle lengths and the quaternion's
+// norm in the reverse pass.
 __device__ __forceinline__ float rsqrt_refined(float x) {
-  const float y = rsqrt_ftz(x);
-  return fmaf(0.5f * y, fmaf(-x * y, y, 1.f), y);
+  const float y = rsqrtf(x), e = fmaf(-x * y, y, 1.f);
+  return fabsf(e) < 1.f ? fmaf(0.5f * y, e, y) : y;
 }
 
 // 16-byte shared-memory accesses (o a multiple of 4).
