@@ -510,20 +510,6 @@ static shac_status upload_model(const shac_model* m, Group& g) {
   return SHAC_OK;
 }
 
-// Lanes per environment chosen for N environments: the fewest that give every
-// link and DOF a lane; below 16, where a component of the subtree sums ([Ic, F] has
-// 16) has no lane of its own, twice as many while the group's warps still fit the
-// GPU at once (8 an SM).  Cart-pole, 64 environments, us a step
-// forward + adjoint: two lanes 41 generic, 18 specialised; sixteen 26 and 15.
-static int default_lanes(const shac_model* m, int N, int num_sms) {
-  const int par = std::max(m->nv, m->L);
-  int lanes = 32;
-  for (int t : {16, 8, 4, 2})
-    if (par <= t) lanes = t;
-  while (lanes < 16 && (int64_t)N * 2 * lanes / 32 <= (int64_t)8 * num_sms) lanes *= 2;
-  return lanes;
-}
-
 // Register row capacity of the batched dense path: the smallest of the device
 // instantiations (2, 4, 6, 8, 10, 12, 14, 16, 20, 24, 28, 32 rows) that holds
 // nv rows, one padded row per lane, when the team has that many lanes; 0
@@ -533,18 +519,63 @@ static int dense_class(int nv, int lanes) {
   return nm <= lanes ? nm : 0;
 }
 
-// Whether group g's team covers its links and DOFs with a lane each
-// (shac_team.cuh) and its records fit the workspace, which is laid out for the
-// general ones (a handful of muscles may not: their items come in whole rows);
-// a batch takes the lane kernels when all its groups do.
+// Whether a wide enough team has the lane form of the model (shac_team.cuh): a
+// lane for every link and DOF, and records that fit the workspace, which is laid
+// out for the general ones (a handful of muscles may not: their items come in
+// whole rows).
+static bool lane_model(const shac_model* m) {
+  return m->lanes_needed <= LANE_COLS && m->lane_layout.rec_floats <= m->layout.rec_floats;
+}
+// Whether group g runs in lane form; a batch takes the lane kernels when all its
+// groups do.
 static bool lane_form(const Group& g) {
-  return g.N == 0 || (g.m->lanes_needed <= g.lanes && dense_class(g.m->nv, g.lanes) > 0 &&
-                      g.m->lane_layout.rec_floats <= g.m->layout.rec_floats);
+  return g.N == 0 || (lane_model(g.m) && g.m->lanes_needed <= g.lanes && dense_class(g.m->nv, g.lanes) > 0);
 }
 static bool lane_form(const shac_batch* b) {
   for (const Group& g : b->groups)
     if (!lane_form(g)) return false;
   return true;
+}
+
+// Default lanes per environment of every group: the fewest that give each link and
+// DOF a lane, so that which kernels a batch takes does not depend on its size.  In
+// the lane form, whose results do not depend on the team size, groups below 16 lanes
+// (where a component of the subtree sums, [Ic, F] has 16, has no lane of its own) take
+// twice as many, the narrowest first, while all groups' warps together still fit the
+// GPU at once (8 an SM).  Cart-pole, 64 environments, us a step forward + adjoint: two
+// lanes 41 generic, 18 specialised; sixteen 26 and 15.
+static std::vector<int> default_lanes(const shac_batch* b) {
+  std::vector<int> lanes;
+  bool widen = true;
+  for (const Group& g : b->groups) {
+    const int par = lane_model(g.m) ? g.m->lanes_needed : std::max(g.m->nv, g.m->L);
+    int n = 32;
+    for (int t : {16, 8, 4, 2})
+      if (par <= t) n = t;
+    lanes.push_back(n);
+    widen = widen && (g.N == 0 || lane_model(g.m));
+  }
+  auto warps = [&](size_t gi) {
+    const int64_t per = 32 / lanes[gi];
+    return (b->groups[gi].N + per - 1) / per;
+  };
+  while (widen) {
+    int64_t total = 0;
+    size_t at = 0;
+    for (size_t gi = 0; gi < lanes.size(); ++gi) {
+      total += warps(gi);
+      if (lanes[gi] < lanes[at]) at = gi;
+    }
+    total -= warps(at);
+    widen = lanes[at] < 16;
+    if (!widen) break;
+    lanes[at] *= 2;
+    if (total + warps(at) > (int64_t)8 * b->num_sms) {
+      lanes[at] /= 2;
+      widen = false;
+    }
+  }
+  return lanes;
 }
 
 // Shared floats per environment: padded so that every environment's scratch
@@ -705,7 +736,6 @@ extern "C" shac_status shac_batch_create(const shac_model* const* models, const 
     Group g;
     g.m = models[gi];
     g.N = n_envs[gi];
-    g.lanes = default_lanes(g.m, g.N, b->num_sms);
     shac_status st = upload_model(g.m, g);
     if (st != SHAC_OK) { shac_batch_destroy(b); return st; }
     GroupIO& io = b->io.g[gi];
@@ -716,6 +746,10 @@ extern "C" shac_status shac_batch_create(const shac_model* const* models, const 
     b->act_size += (int64_t)g.m->na * g.N;
     b->n_envs += g.N;
     b->groups.push_back(g);
+  }
+  {
+    const std::vector<int> lanes = default_lanes(b);
+    for (int gi = 0; gi < n_groups; ++gi) b->groups[gi].lanes = lanes[gi];
   }
   b->io.q_size = b->q_size; b->io.qd_size = b->qd_size; b->io.act_size = b->act_size; b->io.n_envs = b->n_envs;
   std::vector<DevModel> dm;
@@ -766,9 +800,10 @@ extern "C" shac_status shac_batch_set_launch(shac_batch* b, int32_t group, int32
   if (lanes != 0 && lanes != 1 && lanes != 2 && lanes != 4 && lanes != 8 && lanes != 16 && lanes != 32)
     return SHAC_ERR_INVALID_ARG;
   if (warps < 0 || warps > 8) return SHAC_ERR_INVALID_ARG;
+  const std::vector<int> defaults = default_lanes(b);
   for (int gi = 0; gi < (int)b->groups.size(); ++gi) {
     if (group >= 0 && gi != group) continue;
-    b->groups[gi].lanes = lanes == 0 ? default_lanes(b->groups[gi].m, b->groups[gi].N, b->num_sms) : lanes;
+    b->groups[gi].lanes = lanes == 0 ? defaults[gi] : lanes;
   }
   if (warps > 0) b->warps_per_cta = warps;
   return build_items(b);
