@@ -350,8 +350,13 @@ shac_status shac_batch_specialize(shac_batch* batch, int32_t enable);
  * model, h_max = 32, 2048 environments: 2.9 GB; shac_batch_workspace_bytes
  * reports the new size, reallocate after the call).  Contract: the adjoint
  * window must follow the forward window on the same workspace with the same h,
- * q_traj/qd_traj, act (and done mask), with no other window call in between; it
- * then returns what the recomputing adjoint returns, bit for bit.  Step-level
+ * q_traj/qd_traj, act (and done mask), with no other window call (shac_autotune
+ * makes some) on that workspace in between; it then returns what the recomputing adjoint returns,
+ * bit for bit.  The launch shape and the specialisation may change in between
+ * only if the records stay as they are: an adjoint that would read records
+ * written in another form (a team that gained or lost the lane form, kernels
+ * specialised or no longer) returns SHAC_ERR_INVALID_ARG and launches nothing;
+ * go back to the shape of the forward, or run the forward again.  Step-level
  * calls (shac_step, shac_step_adjoint, shac_step_adjoint_static) never use the
  * tape.  keep = 0 (the default) recomputes.  (Sec. 3.1 keeps each substep's
  * Cholesky factor for the backward pass; the tape keeps every intermediate.) */

@@ -1,5 +1,6 @@
 // Host side of the C ABI declared in include/shacsim.h.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -68,8 +69,12 @@ struct shac_batch {
     size_t smem = 0;
     const void* kernel[2] = {nullptr, nullptr};
     unsigned int spec_key = 0;
+    unsigned int records = 0;   // what the substep records look like (never 0)
     int env_stride[MAX_GROUPS] = {0}, dense_nm[MAX_GROUPS] = {0};
   } plan;
+  // records of the last forward window that kept its tape (0: none of this batch yet);
+  // the adjoint reads them with its own layout, so it must be the same
+  std::atomic<unsigned int> tape_records{0};
 };
 
 static shac_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? SHAC_OK : SHAC_ERR_CUDA; }
@@ -635,6 +640,10 @@ static void plan_launch(shac_batch* b) {
     p.smem = (size_t)W * p.smem_warp_floats * sizeof(float);
     const bool spec = b->spec.key != 0u && b->spec_lanes == b->groups[0].lanes;
     if (spec) p.spec_key = b->spec.key;
+    // lane records hold another factor in a specialised build, general ones another
+    // diagonal with the shared-memory dense stages
+    p.records = p.lanes ? (spec ? 2u : 1u) : 3u;
+    for (size_t gi = 0; gi < b->groups.size() && !p.lanes; ++gi) p.records |= (p.dense_nm[gi] > 0 ? 4u : 0u) << gi;
     p.st = SHAC_OK;
     for (int k = 0; k < 2 && p.st == SHAC_OK; ++k) {
       p.kernel[k] = spec ? (k ? b->spec.adj : b->spec.fwd) : batched_kernel(k == 1, p.lanes);
@@ -887,6 +896,11 @@ static shac_status batched_launch(shac_batch* b, BatchedArgs& a, void* ws, cudaS
   a.flags = b->d_flags;
   if (b->n_items == 0) return SHAC_OK;
   if (p.st != SHAC_OK) return p.st;
+  if (a.tape_window) {
+    const unsigned int kept = b->tape_records;
+    if (adjoint && kept != 0u && kept != p.records) return SHAC_ERR_INVALID_ARG;
+    if (!adjoint) b->tape_records = p.records;
+  }
   a.spec_key = p.spec_key;
   const int grid = p.grid[adjoint];
   // a warp for every item: each takes its own, and the shared counter is not needed
@@ -1250,6 +1264,7 @@ extern "C" shac_status shac_autotune(shac_batch* b, void* stream, void* ws, int3
   std::vector<int> lanes0(n_groups), best_lanes(n_groups);
   for (int gi = 0; gi < n_groups; ++gi) lanes0[gi] = best_lanes[gi] = b->groups[gi].lanes;
   const int warps0 = b->warps_per_cta;
+  const unsigned int tape_records0 = b->tape_records;
   int best_warps = warps0;
   float best = INFINITY;
   if (st == SHAC_OK) st = measure(&best);
@@ -1286,6 +1301,7 @@ extern "C" shac_status shac_autotune(shac_batch* b, void* stream, void* ws, int3
   for (int gj = 0; gj < n_groups; ++gj) b->groups[gj].lanes = ok ? best_lanes[gj] : lanes0[gj];
   b->warps_per_cta = ok ? best_warps : warps0;
   const shac_status st_items = build_items(b);
+  b->tape_records = tape_records0;   // the timed windows kept theirs in their own workspace
   cudaStreamSynchronize(s);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);

@@ -49,8 +49,10 @@ class Simulator:
         self._alloc_workspace()
 
     def _alloc_workspace(self):
-        nbytes = int(_lib.load().shac_batch_workspace_bytes(self.batch))
-        self.workspace = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=self.device)
+        nbytes = max(int(_lib.load().shac_batch_workspace_bytes(self.batch)), 256)
+        if getattr(self, "workspace", None) is not None and self.workspace.numel() == nbytes:
+            return    # the size did not change: a kept window tape stays
+        self.workspace = torch.empty(nbytes, dtype=torch.uint8, device=self.device)
         assert self.workspace.data_ptr() % 256 == 0
 
     def __del__(self):
