@@ -77,7 +77,13 @@ struct shac_batch {
   std::atomic<unsigned int> tape_records{0};
 };
 
-static shac_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? SHAC_OK : SHAC_ERR_CUDA; }
+// The status of a CUDA call.  A failure is reported here and nowhere else: the runtime's
+// last error is cleared, so that the launch check of the next call does not find it.
+static shac_status cuda_ok(cudaError_t e) {
+  if (e == cudaSuccess) return SHAC_OK;
+  cudaGetLastError();
+  return SHAC_ERR_CUDA;
+}
 
 // ------------------------------------------------------------------ model --
 
@@ -496,11 +502,11 @@ static shac_status upload_model(const shac_model* m, Group& g) {
   const size_t ibytes = ((iblob.size() * sizeof(int) + 255) / 256) * 256;
   const size_t bytes = ibytes + fblob.size() * sizeof(float);
   char* dev = nullptr;
-  if (cudaMalloc(&dev, bytes) != cudaSuccess) return SHAC_ERR_CUDA;
+  if (cuda_ok(cudaMalloc(&dev, bytes)) != SHAC_OK) return SHAC_ERR_CUDA;
   std::vector<char> host(bytes, 0);
   std::memcpy(host.data(), iblob.data(), iblob.size() * sizeof(int));
   std::memcpy(host.data() + ibytes, fblob.data(), fblob.size() * sizeof(float));
-  if (cudaMemcpy(dev, host.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) { cudaFree(dev); return SHAC_ERR_CUDA; }
+  if (cuda_ok(cudaMemcpy(dev, host.data(), bytes, cudaMemcpyHostToDevice)) != SHAC_OK) { cudaFree(dev); return SHAC_ERR_CUDA; }
   for (auto& f : ifix) *f.first = reinterpret_cast<const int*>(dev) + f.second;
   for (auto& f : ffix) *f.first = reinterpret_cast<const float*>(dev + ibytes) + f.second;
   g.blob = dev;
@@ -650,12 +656,12 @@ static void plan_launch(shac_batch* b) {
       // the opt-in above 48 KB, always to the same limit: other batches launch the
       // same kernels with other sizes
       int occ = 0;
-      if (cudaFuncSetAttribute(p.kernel[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BLOCK_LIMIT) !=
-          cudaSuccess)
+      if (cuda_ok(cudaFuncSetAttribute(p.kernel[k], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)SMEM_BLOCK_LIMIT)) != SHAC_OK)
         p.st = SHAC_ERR_CAPACITY;
-      else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, p.kernel[k], p.block, p.smem) != cudaSuccess)
-        p.st = SHAC_ERR_CUDA;
-      else if (occ < 1)
+      else if ((p.st = cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, p.kernel[k], p.block, p.smem))) ==
+                   SHAC_OK &&
+               occ < 1)
         p.st = SHAC_ERR_CAPACITY;
       p.grid[k] = std::max(1, std::min(b->num_sms * occ, (n_items + W - 1) / W));
     }
@@ -734,8 +740,8 @@ extern "C" shac_status shac_batch_create(const shac_model* const* models, const 
   if (!b) return SHAC_ERR_INVALID_ARG;
   b->form = form;
   b->h_max = window_h_max;
-  if (cudaGetDevice(&b->device) != cudaSuccess ||
-      cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, b->device) != cudaSuccess) {
+  if (cuda_ok(cudaGetDevice(&b->device)) != SHAC_OK ||
+      cuda_ok(cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, b->device)) != SHAC_OK) {
     delete b;
     return SHAC_ERR_CUDA;
   }
@@ -764,15 +770,15 @@ extern "C" shac_status shac_batch_create(const shac_model* const* models, const 
   std::vector<DevModel> dm;
   for (auto& g : b->groups) dm.push_back(g.dev);
   for (auto& g : b->groups) dm.push_back(g.lane_dev);
-  if (cudaMalloc(&b->d_models, dm.size() * sizeof(DevModel)) != cudaSuccess ||
-      cudaMemcpy(b->d_models, dm.data(), dm.size() * sizeof(DevModel), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMalloc(&b->d_flags, sizeof(unsigned int)) != cudaSuccess ||
-      cudaMemset(b->d_flags, 0, sizeof(unsigned int)) != cudaSuccess) {
+  if (cuda_ok(cudaMalloc(&b->d_models, dm.size() * sizeof(DevModel))) != SHAC_OK ||
+      cuda_ok(cudaMemcpy(b->d_models, dm.data(), dm.size() * sizeof(DevModel), cudaMemcpyHostToDevice)) != SHAC_OK ||
+      cuda_ok(cudaMalloc(&b->d_flags, sizeof(unsigned int))) != SHAC_OK ||
+      cuda_ok(cudaMemset(b->d_flags, 0, sizeof(unsigned int))) != SHAC_OK) {
     shac_batch_destroy(b);
     return SHAC_ERR_CUDA;
   }
   b->items_cap = std::max<int64_t>(1, b->n_envs);
-  if (cudaMalloc(&b->d_items, (size_t)b->items_cap * sizeof(WorkItem)) != cudaSuccess) {
+  if (cuda_ok(cudaMalloc(&b->d_items, (size_t)b->items_cap * sizeof(WorkItem))) != SHAC_OK) {
     shac_batch_destroy(b);
     return SHAC_ERR_CUDA;
   }
@@ -836,7 +842,7 @@ extern "C" shac_status shac_batch_specialize(shac_batch* b, int32_t enable) {
   }
   if (b->form != SHAC_FORM_BATCHED || b->groups.size() != 1) return SHAC_ERR_UNSUPPORTED;
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess) return SHAC_ERR_CUDA;
+  if (cuda_ok(cudaGetDevice(&dev)) != SHAC_OK) return SHAC_ERR_CUDA;
   if (dev != b->device) return SHAC_ERR_INVALID_ARG;
   const Group& g = b->groups[0];
   JitKernels k;
@@ -905,7 +911,7 @@ static shac_status batched_launch(shac_batch* b, BatchedArgs& a, void* ws, cudaS
   const int grid = p.grid[adjoint];
   // a warp for every item: each takes its own, and the shared counter is not needed
   if (grid * (p.block / 32) >= b->n_items) a.counter = nullptr;
-  else if (cudaMemsetAsync(a.counter, 0, sizeof(int), s) != cudaSuccess) return SHAC_ERR_CUDA;
+  else if (cuda_ok(cudaMemsetAsync(a.counter, 0, sizeof(int), s)) != SHAC_OK) return SHAC_ERR_CUDA;
   void* args[] = {&a};
   return cuda_ok(cudaLaunchKernel(p.kernel[adjoint], dim3(grid), dim3(p.block), args, p.smem, s));
 }
@@ -945,8 +951,8 @@ static shac_status run_forward(shac_batch* b, cudaStream_t s, void* ws, int h, c
   }
   if (ep) return SHAC_ERR_UNSUPPORTED;
   if (q_copy0) {
-    if (cudaMemcpyAsync(q_copy0, q0, b->q_size * sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync(qd_copy0, qd0, b->qd_size * sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+    if (cuda_ok(cudaMemcpyAsync(q_copy0, q0, b->q_size * sizeof(float), cudaMemcpyDeviceToDevice, s)) != SHAC_OK ||
+        cuda_ok(cudaMemcpyAsync(qd_copy0, qd0, b->qd_size * sizeof(float), cudaMemcpyDeviceToDevice, s)) != SHAC_OK)
       return SHAC_ERR_CUDA;
   }
   for (int gi = 0; gi < (int)b->groups.size(); ++gi) {
@@ -1113,7 +1119,7 @@ static shac_status static_scratch_address(int dev, void** out) {
   std::lock_guard<std::mutex> lock(g_static_mutex);
   if (!g_static_addr[dev]) {
     void* p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return SHAC_ERR_CUDA;
+    if (cuda_ok(cudaGetSymbolAddress(&p, g_static_scratch)) != SHAC_OK || !p) return SHAC_ERR_CUDA;
     g_static_addr[dev] = p;
   }
   *out = g_static_addr[dev];
@@ -1130,7 +1136,7 @@ extern "C" shac_status shac_step_adjoint_static(shac_batch* b, void* stream, con
   // the array used is the current device's: it must be the GPU that holds the
   // batch's model tables and work items
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess) return SHAC_ERR_CUDA;
+  if (cuda_ok(cudaGetDevice(&dev)) != SHAC_OK) return SHAC_ERR_CUDA;
   if (dev != b->device) return SHAC_ERR_INVALID_ARG;
   void* ws = nullptr;
   const shac_status st = static_scratch_address(dev, &ws);
@@ -1143,11 +1149,11 @@ extern "C" shac_status shac_get_status(shac_batch* b, void* stream, uint32_t* fl
   if (!b || !flags) return SHAC_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   unsigned int v = 0;
-  if (cudaMemcpyAsync(&v, b->d_flags, sizeof(v), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
+  if (cuda_ok(cudaMemcpyAsync(&v, b->d_flags, sizeof(v), cudaMemcpyDeviceToHost, s)) != SHAC_OK ||
+      cuda_ok(cudaStreamSynchronize(s)) != SHAC_OK)
     return SHAC_ERR_CUDA;
   *flags = v;
-  if (clear && cudaMemsetAsync(b->d_flags, 0, sizeof(unsigned int), s) != cudaSuccess) return SHAC_ERR_CUDA;
+  if (clear && cuda_ok(cudaMemsetAsync(b->d_flags, 0, sizeof(unsigned int), s)) != SHAC_OK) return SHAC_ERR_CUDA;
   return (v & FLAG_NONFINITE) ? SHAC_ERR_NONFINITE : SHAC_OK;
 }
 
@@ -1250,10 +1256,10 @@ extern "C" shac_status shac_autotune(shac_batch* b, void* stream, void* ws, int3
     if (r != SHAC_OK) return r;
     float t[3];
     for (int rep = 0; rep < 3; ++rep) {
-      if (cudaEventRecord(e0, s) != cudaSuccess) return SHAC_ERR_CUDA;
+      if (cuda_ok(cudaEventRecord(e0, s)) != SHAC_OK) return SHAC_ERR_CUDA;
       if ((r = window()) != SHAC_OK) return r;
-      if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess) return SHAC_ERR_CUDA;
-      if (cudaEventElapsedTime(&t[rep], e0, e1) != cudaSuccess) return SHAC_ERR_CUDA;
+      if (cuda_ok(cudaEventRecord(e1, s)) != SHAC_OK || cuda_ok(cudaEventSynchronize(e1)) != SHAC_OK) return SHAC_ERR_CUDA;
+      if (cuda_ok(cudaEventElapsedTime(&t[rep], e0, e1)) != SHAC_OK) return SHAC_ERR_CUDA;
     }
     std::sort(t, t + 3);
     *ms = t[1];
