@@ -239,7 +239,6 @@ static void compute_layout(shac_model* m) {
   d.rec_floats = o;
   take(d.o_ACT, m->na); take(d.o_QB, m->nq); take(d.o_QDB, nv); take(d.o_ACTB, m->na);
   take(d.o_QC, m->nq); take(d.o_QDC, nv); take(d.o_LW, LWORK * L);
-  d.lanes_needed = m->lanes_needed;
   d.nround = m->nround;
   d.deepest = m->deepest;
   d.mrows = m->mrows;
@@ -266,7 +265,6 @@ static void compute_layout(shac_model* m) {
   o = 0;
   take(l.o_Q, m->nq); take(l.o_QD, nv); take(l.o_ACT, m->na); take(l.o_QB, m->nq); take(l.o_QDB, nv);
   take(l.o_ACTB, m->na);
-  take(l.o_QC, m->nq); take(l.o_QDC, nv);
   if (m->nseg > 0) {
     take(l.o_SEGA, m->nseg); take(l.o_MW, 12 * MSLOTS); take(l.o_MB, 6 * L);
     o = (o + 3) / 4 * 4;
@@ -513,10 +511,9 @@ static shac_status upload_model(const shac_model* m, Group& g) {
   g.lane_dev = g.dev;   // the same arrays under the lane form's offsets
   const DevModel& l = m->lane_layout;
   int DevModel::*const offsets[] = {&DevModel::o_Q, &DevModel::o_QD, &DevModel::o_ACT, &DevModel::o_QB, &DevModel::o_QDB,
-                                    &DevModel::o_ACTB, &DevModel::o_QC, &DevModel::o_QDC, &DevModel::o_SEGA,
-                                    &DevModel::o_MW, &DevModel::o_X, &DevModel::o_R, &DevModel::o_MP, &DevModel::o_MB,
-                                    &DevModel::o_MX, &DevModel::o_MF, &DevModel::rec_floats,
-                                    &DevModel::env_floats};
+                                    &DevModel::o_ACTB, &DevModel::o_SEGA, &DevModel::o_MW, &DevModel::o_X,
+                                    &DevModel::o_R, &DevModel::o_MP, &DevModel::o_MB, &DevModel::o_MX,
+                                    &DevModel::o_MF, &DevModel::rec_floats, &DevModel::env_floats};
   for (int DevModel::*f : offsets) g.lane_dev.*f = l.*f;
   return SHAC_OK;
 }
@@ -672,7 +669,6 @@ static void plan_launch(shac_batch* b) {
 
 // Work items sorted by per-warp cost (largest first) so the dynamic schedule
 // finishes the long items early.
-static void plan_launch(shac_batch* b);
 static shac_status build_items(shac_batch* b) {
   plan_launch(b);
   std::vector<std::pair<double, WorkItem>> items;

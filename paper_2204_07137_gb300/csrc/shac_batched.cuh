@@ -108,7 +108,7 @@ __device__ __forceinline__ void forward_item(const BatchedArgs& a, const DevMode
                                : nullptr;
   for (int step = 0; step < a.h; ++step) {
     team_load(w, M.o_ACT, a.act + (size_t)step * a.io.act_size + io.act_off, M.na, io.N, t.env, t.lane, t.nl);
-    clear_comp(M, w, t.lane, t.nl);
+    if (!LANES) clear_comp(M, w, t.lane, t.nl);   // the lane form's are registers
     team_sync(t.nl);
     float* wt = wtape ? wtape + (size_t)step * a.tape_step[it.group] : nullptr;
     if (LANES) {
@@ -199,7 +199,7 @@ __device__ __forceinline__ void adjoint_item(const BatchedArgs& a, const DevMode
       zero_range(w, M.o_QB, M.nq, t.lane, t.nl);
       zero_range(w, M.o_QDB, M.nv, t.lane, t.nl);
     }
-    clear_comp(M, w, t.lane, t.nl);
+    if (!LANES) clear_comp(M, w, t.lane, t.nl);
     team_sync(t.nl);
     const float* recs = tape;   // this step's substep records
     if (a.tape_window) {        // kept by the forward window: the post-step state is read back

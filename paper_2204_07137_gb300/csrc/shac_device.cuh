@@ -95,10 +95,9 @@ struct DevModel {
   const float *fmax;
   // reward weights
   const float *rwq, *rwqd;
-  // lane form (shac_team.cuh): lanes a team needs (DOFs, then the links without
-  // one), doubling rounds, the deepest link's level, and the lane columns of the
-  // model's constants
-  int lanes_needed, nround, deepest;
+  // lane form (shac_team.cuh): doubling rounds, the deepest link's level, and the lane
+  // columns of the model's constants
+  int nround, deepest;
   signed char par8[32];                  // link parents (models of at most 32 links)
   const int* ln_i;
   const float* ln_f;
@@ -1480,13 +1479,12 @@ __device__ __forceinline__ void lk_adj_local(const DevModel& M, const Mem& w, in
 
 // Reverse of one muscle segment: cotangents of both via points and of the
 // activation (stored per segment).
-// x0, x1: the segment's via points, f0 the force on the first (its negative on
-// the second).
 template <class Mem>
-__device__ __forceinline__ void seg_adjoint(const DevModel& M, const Mem& w, int sg, V3 x0, V3 f0, V3 x1) {
+__device__ __forceinline__ void seg_adjoint(const DevModel& M, const Mem& w, int sg) {
   const int e0 = M.nc + 2 * sg, e1 = e0 + 1;
   const int l0 = __ldg(M.item_link + e0), l1 = __ldg(M.item_link + e1);
-  const V3 f1 = -f0;
+  const V3 x0 = ld3(w, M.o_IT + 7 * e0), f0 = ld3(w, M.o_IT + 7 * e0 + 3);
+  const V3 x1 = ld3(w, M.o_IT + 7 * e1), f1 = ld3(w, M.o_IT + 7 * e1 + 3);
   const V3 n0b = -ld3(w, lwork(M, l0) + LW_FB), f0eb = -ld3(w, lwork(M, l0) + LW_FB + 3);
   const V3 n1b = -ld3(w, lwork(M, l1) + LW_FB), f1eb = -ld3(w, lwork(M, l1) + LW_FB + 3);
   const V3 f0b = cross(n0b, x0) + f0eb, f1b = cross(n1b, x1) + f1eb;
@@ -1508,34 +1506,6 @@ __device__ __forceinline__ void seg_adjoint(const DevModel& M, const Mem& w, int
   w[M.o_SEGA + sg] = (araw > 0.f && araw < 1.f) ? Fb * fm : 0.f;
   st3(w, M.o_ITB + 10 * e0, x0b);
   st3(w, M.o_ITB + 10 * e1, x1b);
-}
-
-// After every segment: the activations' cotangents (into o_ACTB) and each
-// link's via-point pose cotangents in `parts` partial sums (o_MW).
-template <class Mem>
-__device__ __forceinline__ void muscle_adj_gather(const DevModel& M, const Mem& w, int lane, int nl) {
-  for (int mu_ = lane; mu_ < M.nm; mu_ += nl) {
-    float sa = 0.f;
-    for (int sg = __ldg(M.mus_seg_ptr + mu_); sg < __ldg(M.mus_seg_ptr + mu_ + 1); ++sg) sa += w[M.o_SEGA + sg];
-    w[M.o_ACTB + M.ntact + mu_] += sa;
-  }
-  const int parts = muscle_parts(M, nl);
-  for (int sl = lane; sl < M.L * parts; sl += nl) {
-    const int i = sl / parts, r = sl % parts;
-    V3 Pb = v3(0.f, 0.f, 0.f);
-    M33 Rb;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) Rb.m[k] = 0.f;
-    for (int k = __ldg(M.lm_ptr + i) + r; k < __ldg(M.lm_ptr + i + 1); k += parts) {
-      const int e = __ldg(M.lm_idx + k);
-      const V3 xb = ld3(w, M.o_ITB + 10 * e);
-      Pb = Pb + xb;
-      add_outer(Rb, xb, cld3(M.item_pos + 3 * e));
-    }
-    st3(w, M.o_MW + 12 * sl, Pb);
-    stm(w, M.o_MW + 12 * sl + 3, Rb);
-  }
-  team_sync(nl);
 }
 
 // Children's contributions carried up a chain in registers: subtree sums of
@@ -1821,13 +1791,32 @@ __device__ __forceinline__ void st_dynamics_adj(const DevModel& M, const Mem& w,
   for (int d = nl - 1 - lane; d < M.nv; d += nl) dof_adj_force(M, w, d);
   team_sync(nl);
   if (M.nseg > 0) {
-    for (int sg = lane; sg < M.nseg; sg += nl) {
-      const int e = M.o_IT + 7 * (M.nc + 2 * sg);
-      seg_adjoint(M, w, sg, ld3(w, e), ld3(w, e + 3), ld3(w, e + 7));
+    for (int sg = lane; sg < M.nseg; sg += nl) seg_adjoint(M, w, sg);
+    team_sync(nl);
+    for (int mu_ = lane; mu_ < M.nm; mu_ += nl) {
+      float sa = 0.f;
+      for (int sg = __ldg(M.mus_seg_ptr + mu_); sg < __ldg(M.mus_seg_ptr + mu_ + 1); ++sg) sa += w[M.o_SEGA + sg];
+      w[M.o_ACTB + M.ntact + mu_] += sa;
+    }
+    // each link's via-point pose cotangents in `parts` partial sums, then
+    // added in part order
+    const int parts = muscle_parts(M, nl);
+    for (int sl = lane; sl < M.L * parts; sl += nl) {
+      const int i = sl / parts, r = sl % parts;
+      V3 Pb = v3(0.f, 0.f, 0.f);
+      M33 Rb;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) Rb.m[k] = 0.f;
+      for (int k = __ldg(M.lm_ptr + i) + r; k < __ldg(M.lm_ptr + i + 1); k += parts) {
+        const int e = __ldg(M.lm_idx + k);
+        const V3 xb = ld3(w, M.o_ITB + 10 * e);
+        Pb = Pb + xb;
+        add_outer(Rb, xb, cld3(M.item_pos + 3 * e));
+      }
+      st3(w, M.o_MW + 12 * sl, Pb);
+      stm(w, M.o_MW + 12 * sl + 3, Rb);
     }
     team_sync(nl);
-    muscle_adj_gather(M, w, lane, nl);   // added below in part order
-    const int parts = muscle_parts(M, nl);
     for (int i = lane; i < M.L; i += nl) {
       V3 Pb = v3(0.f, 0.f, 0.f);
       M33 Rb;

@@ -52,7 +52,7 @@ const Field kFields[] = {
     {"o_ITB", &DevModel::o_ITB}, {"o_SEGA", &DevModel::o_SEGA}, {"o_MW", &DevModel::o_MW},
     {"o_RDB", &DevModel::o_RDB}, {"o_X", &DevModel::o_X}, {"o_R", &DevModel::o_R},
     {"o_MP", &DevModel::o_MP}, {"o_MB", &DevModel::o_MB}, {"o_MX", &DevModel::o_MX}, {"o_MF", &DevModel::o_MF},
-    {"mrows", &DevModel::mrows}, {"lanes_needed", &DevModel::lanes_needed},
+    {"mrows", &DevModel::mrows},
     {"nround", &DevModel::nround}, {"deepest", &DevModel::deepest}, {"rec_floats", &DevModel::rec_floats}, {"env_floats", &DevModel::env_floats},
 };
 
@@ -81,9 +81,9 @@ std::string mask_list(const std::vector<int>& masks) {
 }
 
 std::string spec_string(int device, const DevModel& m, const std::vector<int>& parent, const std::vector<int>& masks,
-                        int lanes, int rows, int stride) {
+                        int lanes, int rows, int stride, bool lane_form) {
   std::string s = "dev" + std::to_string(device) + ";lanes" + std::to_string(lanes) + ";rows" +
-                  std::to_string(rows) + ";stride" + std::to_string(stride);
+                  std::to_string(rows) + ";stride" + std::to_string(stride) + (lane_form ? ";lane form" : ";general");
   for (const Field& f : kFields) s += ";" + std::string(f.name) + "=" + std::to_string(m.*(f.member));
   return s + ";parents=" + parent_list(parent) + ";masks=" + mask_list(masks);
 }
@@ -103,7 +103,7 @@ std::map<std::string, JitKernels> g_cache;
 shac_status jit_kernels(int device, const DevModel& m, const std::vector<int>& parent, const std::vector<int>& masks,
                         int lanes, int rows, int stride, bool lane_form, JitKernels* out, std::string* log) {
   if ((int)parent.size() != m.L) return SHAC_ERR_INVALID_ARG;
-  const std::string spec = spec_string(device, m, parent, masks, lanes, rows, stride);
+  const std::string spec = spec_string(device, m, parent, masks, lanes, rows, stride, lane_form);
   std::lock_guard<std::mutex> lock(g_mutex);
   auto it = g_cache.find(spec);
   if (it != g_cache.end()) { *out = it->second; return SHAC_OK; }

@@ -612,7 +612,7 @@ __device__ __forceinline__ void si_mul(const float (&si)[10], V3 xw, V3 xv, V3& 
           sum3(si[8], xw.x, si[9], xw.y, si[6], xw.z)) + cross(h, xv);
   yf = si[0] * xv - cross(h, xw);
 }
-__device__ __forceinline__ void lane_local(const DevModel& M, const SMem& w, const LaneConst& c, float zroot,
+__device__ __forceinline__ void lane_local(const DevModel& M, const LaneConst& c, float zroot,
                                            LaneLink& k) {
   const V3 cm = k.P + mul(k.R, c.com);
   M33 Ic;
@@ -879,7 +879,7 @@ __device__ __forceinline__ void lane_substep(const DevModel& M, const SMem& w, c
   k.av = cross(k.Vw, uv) + cross(k.Vv, uw);
   k.av = k.av + c.base;
   path_sums(M, c, nl, k.aw, k.av);
-  lane_local(M, w, c, c.on_root ? s.rq[2] : 0.f, k);
+  lane_local(M, c, c.on_root ? s.rq[2] : 0.f, k);
   const bool link = c.link >= 0;
   if (M.nseg > 0) {   // muscles: a segment spans two links, so the poses go through memory
     muscle_put_pose(M, w, c.link, k.R, k.P);
