@@ -29,10 +29,10 @@
 // What bounds it is latency: at 2048 environments an SM holds seven warps, so a
 // substep costs its dependent instructions, not its arithmetic.  The per-link
 // passes over shared-memory scratch that this form replaces cost a store, a
-// barrier and a load between any two of them.  Measured on the ant-like model,
-// specialised, a substep's cycles (T = 16): forward 10.8 k -> 4.6 k, reverse
-// 11.5 k -> 5.0 k; forward + adjoint of 2048 environments, h = 8: 2.09 -> 1.00 ms;
-// the generic kernels on 1531 environments, h = 2: 0.98 -> 0.48 ms.
+// barrier and a load between any two of them.  Measured on the ant-like model:
+// specialised, 2048 environments, h = 8, forward + adjoint 2.09 -> 1.01 ms (a substep's
+// cycles at T = 16, before the roundings above: forward 10.8 k -> 4.4 k, reverse
+// 11.5 k -> 5.0 k); the generic kernels on 1531 environments, h = 2: 0.99 -> 0.47 ms.
 #pragma once
 #include "shac_device.cuh"
 
@@ -130,10 +130,11 @@ __device__ __forceinline__ void path_sums(const DevModel& M, const LaneConst& c,
 
 // 1 / sqrt(x): rsqrtf (documented maximum error 2 ulp) and one Newton step of
 // y -> y (3 - x y^2) / 2, to a relative error below 1.5 * 2^-24; 0 gives infinity and
-// infinity 0, where the step has no value.  Serves muscle lengths and the quaternion's
-// norm in the reverse pass: 200 environments of the 152-muscle model, specialised,
-// h = 3, take 0.71 ms forward and 1.47 ms back with it, 0.73 and 1.56 ms with
-// 1.f / sqrtf(x) for the lengths.
+// infinity 0, where the step has no value.  Serves muscle lengths and, in the reverse
+// pass, sliding speeds and the quaternion's norm.  200 environments of the 152-muscle
+// model, specialised, h = 3, take 0.71 ms forward and 1.47 ms back with it, 0.73 and
+// 1.56 ms with 1.f / sqrtf(x) for the lengths; the ant-like model's window on the ground
+// 0.73 ms back with it and 0.75 with 1.f / sqrtf(x) for the speeds (1531, h = 8).
 __device__ __forceinline__ float rsqrt_refined(float x) {
   const float y = rsqrtf(x), e = fmaf(-x * y, y, 1.f);
   return fabsf(e) < 1.f ? fmaf(0.5f * y, e, y) : y;
@@ -1193,7 +1194,7 @@ __device__ __forceinline__ void lane_reverse(const DevModel& M, const SMem& w, c
       const V3 vp = k.Vv + cross(k.Vw, x);
       const float fn = (-M.ke + M.kd * vp.z) * dep;
       const bool slow = (on & 2u) != 0u;
-      const float iv = slow ? 0.f : 1.f / sqrtf(sum2(vp.x, vp.x, vp.y, vp.y));   // 1 / |v_t|
+      const float iv = slow ? 0.f : rsqrt_refined(sum2(vp.x, vp.x, vp.y, vp.y));   // 1 / |v_t|
       const float fmax = M.mu * fabsf(fn);
       const V3 neb = -nb;
       const V3 fbar = cross(neb, x) - fb;
