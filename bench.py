@@ -86,10 +86,10 @@ def algo_bytes_per_env_step(model):
 # kernels on the full ant-2048 h = 32 window, from a one-pass ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum of one launch of each kernel);
 # None where no capture of the current kernels exists.  The recomputing
-# adjoint's traffic is mostly its per-step substep records (about 91 MB per
+# adjoint's traffic is mostly its per-step substep records (about 82 MB per
 # step for 2048 environments) written back from L2 as they are replaced step
 # after step.
-TRAFFIC_BYTES_PER_LAUNCH = {"ant-2048": {"forward": 2.407168e6 + 0.0, "adjoint_recompute": 201.74336e6 + 2316.516608e6,
+TRAFFIC_BYTES_PER_LAUNCH = {"ant-2048": {"forward": 2.40e6 + 0.0, "adjoint_recompute": 28.18e6 + 1.68e9,
                                          "adjoint_tape": None}}
 
 

@@ -23,8 +23,8 @@
 // decided by rounding; with other roundings one of some 80,000 environments came out
 // with a gradient some percent off the general kernels' (2 % of the batches of 1531
 // ant-like environments over two steps), with the same roundings none.  It costs the
-// generic windows about a tenth (1531 environments, h = 8: 1.67 -> 1.84 ms; the general
-// kernels 3.97; the deeper humanoid-like model 7.3 -> 8.8; 19.8).
+// generic windows about a tenth (1531 environments, h = 8: 1.67 -> 1.78 ms; the general
+// kernels 3.97; 512 of the deeper humanoid-like model 7.3 -> 8.8; 19.8).
 //
 // What bounds it is latency: at 2048 environments an SM holds seven warps, so a
 // substep costs its dependent instructions, not its arithmetic.  The per-link
